@@ -158,7 +158,7 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-KSRC = {"k_bfs": "k_bfs.cu", "k_pfm_cta": "k_pfm_cta.cu", "k_pfm": "k_pfm.cu"}
+KSRC = {"k_hop": "k_hop.cu", "k_bfs": "k_bfs.cu", "k_pfm_cta": "k_pfm_cta.cu", "k_pfm": "k_pfm.cu"}
 
 
 def kernel_source_digest(kernel: str):
@@ -287,9 +287,9 @@ def kernel_rooflines(info, opt, peak, ms=None):
         out["k_pfm_cta"]["frac"] = out["k_pfm_cta"]["achieved"] / peak
         out["k_pfm_cta"]["frac_own_model"] = out["k_pfm_cta"]["achieved_own_model"] / peak
     else:
-        out["k_bfs"] = {"achieved": info["alg_bytes"] / (ms / 1e3) / 1e9, "alg_bytes": info["alg_bytes"], "ms": ms,
+        out["k_hop"] = {"achieved": info["alg_bytes"] / (ms / 1e3) / 1e9, "alg_bytes": info["alg_bytes"], "ms": ms,
                         "launches": info["search_launches"]}
-        out["k_bfs"]["frac"] = out["k_bfs"]["achieved"] / peak
+        out["k_hop"]["frac"] = out["k_hop"]["achieved"] / peak
     for k in out:
         tr = recorded_traffic(k + "@large", out[k]["alg_bytes"] / max(1, out[k]["launches"]))
         out[k]["traffic_per_launch"] = tr
@@ -641,7 +641,7 @@ def main():
 
     # dominant kernel: search time per optimality family (sequential pass)
     pfm_kernel = "k_pfm" if os.environ.get("MANTRA_PFM_KERNEL") == "lane" else "k_pfm_cta"
-    fam = {k: tuple(o for o in v_ if o in OPTS) for k, v_ in {"k_bfs": ("sh", "sfm"), pfm_kernel: ("pfm",)}.items()}
+    fam = {k: tuple(o for o in v_ if o in OPTS) for k, v_ in {"k_hop": ("sh", "sfm"), pfm_kernel: ("pfm",)}.items()}
     fam = {k: v_ for k, v_ in fam.items() if v_}
     kms = {k: sum(st[o]["kernel_ms"] for st in seq_infos for o in os_) for k, os_ in fam.items()}
     kbytes = {k: sum(st[o]["alg_bytes"] for st in seq_infos for o in os_) for k, os_ in fam.items()}

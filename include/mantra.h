@@ -224,9 +224,9 @@ int mantra_estimate_batch(mantra_problem* probs, uint32_t count);
  * search kernels on probes -- fixed-r estimates of the graph itself, one per
  * candidate and the same seed for all, each timed by the library's CUDA events
  * -- and keeps the fastest for that graph:
- *   sh / sfm (k_bfs): CTA size 256, 512 or 1024 threads (how many samples run
- *     at once per SM, and the frontier tile a CTA scans per pass) x the
- *     visited bitmap in shared or in global memory (shared only where it fits);
+ *   sh / sfm (k_hop): CTA size 256, 512 or 1024 threads (how many samples run
+ *     at once per SM, and the vertices a CTA takes per pass) x the next level's
+ *     arrivals in shared or in global memory (shared only where they fit);
  *   pfm (CTA kernel): CTA size 256 or 512 x the arrival state in shared
  *     memory (as 32-bit arrival slots, or as 16-bit offsets within each
  *     vertex's slots when no vertex has more than 65,534 slots), in global
@@ -236,13 +236,12 @@ int mantra_estimate_batch(mantra_problem* probs, uint32_t count);
  * kernel time by a calibration run of the defaults, between 8 and 64 samples
  * per SM.  Every candidate runs within the same workspace, whose size is bounded by
  * the engine's share of free device memory.  Later calls whose largest graph
- * of that kernel family is g use g's choice (ticks of small bootstraps keep
- * their 1024-thread shape).  Results never depend on the choice: sample i
+ * of that kernel family is g use g's choice.  Results never depend on the choice: sample i
  * draws from Philox counters fixed by (seed, i).  Call it before sharing g
  * between threads; a tuned graph can be tuned again. */
 typedef struct {
     uint32_t bfs_threads;        /* chosen sh/sfm CTA size */
-    uint32_t bfs_bitmap_shared;  /* 1: the visited bitmap in shared memory */
+    uint32_t bfs_bitmap_shared;  /* 1: the per-vertex search state in shared memory */
     uint32_t pfm_threads;        /* chosen pfm CTA size */
     uint32_t pfm_state_shared;   /* 1: the arrival state in shared memory */
     uint32_t bfs_resident_ctas;  /* samples in flight of the choice (resident CTAs) */
@@ -327,10 +326,9 @@ int mantra_sample_paths_noalloc(const mantra_graph* g, mantra_opt opt, uint64_t 
  * family) plus the search workspaces shared by all, sized for the largest
  * graph of each search family (sh/sfm; pfm) among them, counted for four
  * (sh/sfm) or six (pfm) CTAs per SM (per CTA about 28 bytes per arrival
- * slot and 28 per node for sh/sfm, 44 and 52 with the ob / RTB scratch; 56
- * per node plus 4 per unit of the graph's path-count bound for pfm), and
- * fewer than
- * `max_active` (0 = 256) run; a request is always admitted when none is
+ * slot and 28 per node for sh/sfm, at least 10 and 70 with small graphs' path
+ * sets; with RTB or fsfm requests also 44 and 52; 56 per node plus 4 per unit
+ * of the graph's path-count bound for pfm), and fewer than `max_active` (0 = 256) run; a request is always admitted when none is
  * running.  Each tick launches the pending samples of every running request
  * together; finished requests leave between ticks and queued ones join at the
  * next tick.  A request's result equals mantra_estimate on the same

@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <condition_variable>
 #include <deque>
@@ -29,7 +30,7 @@ using namespace mantra;
 // leave the engine's defaults.
 struct Knobs {
     int bfs_nt = 0;      // sh/sfm CTA size: 256, 512 or 1024
-    int bfs_smem = -1;   // visited bitmap: 1 shared memory, 0 global
+    int bfs_smem = -1;   // first slots of the next level: 1 shared memory, 0 global
     int pfm_nt = 0;      // pfm CTA size: 256 or 512
     int pfm_mode = -1;   // pfm arrival state: 1 shared memory, 0 global, 2 global with the out-edge tiles
                          // staged in shared memory by bulk copies
@@ -80,6 +81,21 @@ int upload_store(const StoreHost& H, mantra_graph* G, cudaStream_t st) {
     dst[SA_OUT_LOFF] = &loff_words;
     size_t total = 0;
     for (int k = 0; k < SA_COUNT; ++k) total += al256((H.len[k] + 1) * 4);
+    // filled on the device: the edges' head and continuation, the in-edges' out-CSR
+    // index, the edges' usable slots, and the out-rows cut at up to 32 times (as many as the mean row has
+    // edges, so that the directory is no larger than the edge arrays)
+    uint32_t nb = 1;
+    while (nb < 32 && (uint64_t)nb * H.n < H.m) nb *= 2;
+    const size_t o_vn = total;
+    total += al256(((size_t)H.m + 1) * 8);
+    const size_t o_io = total;
+    total += al256(((size_t)H.m + 1) * 4);
+    const size_t o_pe = total;
+    total += al256(((size_t)H.m + 1) * 4);
+    const size_t o_dir = total;
+    total += al256((size_t)nb * H.n * 8);
+    const size_t o_dt = total;
+    total += al256(32 * 4);
     if (cudaMalloc(&G->dmem, total) != cudaSuccess) return MANTRA_E_NOMEM;
     size_t off = 0;
     for (int k = 0; k < SA_COUNT; ++k) {
@@ -88,6 +104,19 @@ int upload_store(const StoreHost& H, mantra_graph* G, cudaStream_t st) {
         *dst[k] = (const uint32_t*)p;
         off += al256((H.len[k] + 1) * 4);
     }
+    uint32_t dt[32] = {};
+    for (uint32_t j = 1; j < nb; ++j) dt[j] = H.arr[SA_ST_T][(size_t)j * H.m / nb];   // m > n here
+    char* base = (char*)G->dmem;
+    CU(cudaMemcpyAsync(base + o_dt, dt, sizeof dt, cudaMemcpyHostToDevice, st));
+    G->dg.n = H.n; G->dg.m = H.m; G->dg.A = H.A;
+    G->dg.out_vn = (const uint2*)(base + o_vn);
+    G->dg.in_out = (const uint32_t*)(base + o_io);
+    G->dg.out_pend = (const uint32_t*)(base + o_pe);
+    G->dg.dir = (const uint2*)(base + o_dir);
+    G->dg.dir_t = (const uint32_t*)(base + o_dt);
+    G->dg.dir_n = nb;
+    CU(launch_edge_maps(G->dg, (uint2*)(base + o_vn), (uint32_t*)(base + o_io), (uint32_t*)(base + o_pe),
+                        (uint2*)(base + o_dir), st));
     CU(cudaStreamSynchronize(st));
     G->dg.out_loff = reinterpret_cast<const unsigned short*>(loff_words);
     G->n = H.n; G->m = H.m; G->A = H.A; G->n_uedge = H.n_uedge;
@@ -208,11 +237,19 @@ struct Engine {
     char* bfs_mem = nullptr; BfsWs bws{}; size_t bfs_smem = 0; uint32_t bfs_n = 0, bfs_A = 0, bfs_z = 0;
     int bfs_grids[3][2] = {};
     int bfs_rule_smem = 0;     // default placement: shared only while it keeps the 512-thread residency
-    int bfs_grid = 0;          // resident CTAs of the default (512 threads, default placement)
     bool bfs_dl = false;       // the regions carry the ob / RTB scratch
-    int tick_bfs_nt = 512;     // sh/sfm CTA size of the current tick
+    int tick_bfs_nt = 512;     // k_bfs CTA size of the current tick
     int tick_bfs_sm = 0;       // its bitmap placement
-    bool tick_frac = false;    // the tick has an ob or RTB problem on the sh/sfm kernel
+    // sh/sfm level search (k_hop): regions for the largest resident grid (256
+    // threads, arrivals in global memory); shapes 0 = 256, 1 = 512, 2 = 1024
+    // threads; the arrivals in shared memory are sized by the tick's graphs
+    // (hop_nsm: their largest node count, rounded up)
+    char* hop_mem = nullptr; HopWs hws{}; uint32_t hop_n = 0, hop_A = 0;
+    int hop_regions = 0;
+    std::map<uint64_t, int> hop_occ;       // (shape, shared nodes) -> CTAs per SM
+    int tick_hop_nt = 256, tick_hop_sm = 0, tick_hop_cls = 0;
+    uint32_t tick_hop_n = 0;
+    bool tick_b = false, tick_h = false, tick_p = false;   // kernel families with samples in the current tick
     char* pfm_mem = nullptr; PfmWs pws{}; int pfm_grid = 0; uint32_t pfm_n = 0, pfm_lcap = 0; uint64_t pfm_warps = 0;
     // pfm, one CTA per sample: shapes 0 = 256, 1 = 512 threads; modes 0 = state
     // in global memory, 1 = in shared memory, 2 = global with staged edge tiles,
@@ -226,7 +263,7 @@ struct Engine {
     uint32_t cap = 0;
     char* tab_h = nullptr; char* tab_d = nullptr; size_t tab_bytes = 0;
     char* slot_h = nullptr; char* slot_d = nullptr;
-    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_ri = 0, o_rs = 0;
+    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_uh = 0, o_th = 0, o_ri = 0, o_rs = 0;
     int red_grid = 0;
     // captured ticks, by launch configuration (tick_key)
     std::map<int, cudaGraphExec_t> gexec;
@@ -264,12 +301,16 @@ struct Engine {
     static int shape_of(int nt) { return nt == 256 ? 0 : (nt == 1024 ? 2 : 1); }
 
     int tick_key() const {
-        return (tick_cta ? 1 : 0) | (shape_of(tick_bfs_nt) << 1) | (tick_bfs_sm << 3) | ((tick_frac ? 1 : 0) << 4) |
-               ((tick_pc_nt == 256 ? 0 : 1) << 5) | (tick_pc_sm << 6);   // tick_pc_sm: the pfm mode (2 bits)
+        // a family without samples is not launched; its launch choices are left out
+        int key = (tick_b ? 1 : 0) | (tick_h ? 2 : 0) | (tick_p ? 4 : 0);
+        if (tick_b) key |= (shape_of(tick_bfs_nt) << 3) | (tick_bfs_sm << 5);
+        if (tick_h) key |= (shape_of(tick_hop_nt) << 6) | (tick_hop_sm << 8) | ((tick_hop_sm ? tick_hop_cls : 0) << 13);
+        if (tick_p) key |= ((tick_cta ? 1 : 0) << 9) | ((tick_pc_nt == 256 ? 0 : 1) << 10) | (tick_pc_sm << 11);
+        return key;
     }
 
-    // Table block layout: header | 2 work counters | unit starts (bfs, pfm) |
-    // tasks (bfs, pfm) | reduction items | reduction row starts.
+    // Table block layout: header | work counters | unit starts (bfs, pfm, hop) |
+    // tasks (bfs, pfm, hop) | reduction items | reduction row starts.
     int ensure_tables(uint32_t need) {
         if (tab_h && need <= cap) return MANTRA_OK;
         uint32_t nc = std::max<uint32_t>(64, cap);
@@ -280,11 +321,13 @@ struct Engine {
         if (slot_d) { cudaFree(slot_d); slot_d = nullptr; }
         size_t o = 0;
         o_hdr = o;  o = al256(o + 16);
-        o_work = o; o = al256(o + 16);
+        o_work = o; o = al256(o + 24);
         o_ub = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_up = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_tb = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_tp = o;   o = al256(o + (size_t)nc * sizeof(Task));
+        o_uh = o;   o = al256(o + (size_t)(nc + 1) * 8);
+        o_th = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_ri = o;   o = al256(o + (size_t)nc * sizeof(ReduceItem));
         o_rs = o;   o = al256(o + (size_t)(nc + 1) * 4);
         tab_bytes = o;
@@ -298,22 +341,69 @@ struct Engine {
         return MANTRA_OK;
     }
 
-    // sh/sfm: one region per resident CTA of the largest grid over CTA shapes
-    // and bitmap placements, at most 60 % of free memory.  Every region holds
-    // a global visited bitmap as well, so the placement is chosen per launch.
     // Device bytes of the search workspaces for graphs with these maxima (sh/sfm:
-    // n, A, slots per vertex, ob/RTB scratch; pfm: n, cbound), at the largest
-    // grid of any CTA shape (256-thread CTAs: four per SM for k_bfs, six for
-    // k_pfm_cta) and without the free-memory caps of ensure_bfs /
-    // ensure_pfm_cta: an upper estimate of what those allocate.
-    size_t ws_estimate(uint32_t n, uint32_t A, uint32_t zc, bool dl, uint32_t pn, uint32_t cb) const {
+    // n, A, slots per vertex; with full also k_bfs, which RTB and fsfm run on,
+    // and its RTB scratch; pfm: n, cbound), at the largest grid of any CTA shape
+    // (256-thread CTAs: four per SM for k_hop and k_bfs, six for k_pfm_cta) and
+    // without the free-memory caps of ensure_hop / ensure_bfs / ensure_pfm_cta:
+    // an upper estimate of what those allocate.
+    size_t ws_estimate(uint32_t n, uint32_t A, uint32_t zc, bool full, uint32_t pn, uint32_t cb) const {
         size_t b = 0;
         const size_t sms = (size_t)std::max(num_sms, 1);
-        if (n) { BfsWs w{}; b += 4 * sms * bfs_region_bytes(n, A, zc, false, dl, &w); }
+        if (n) {
+            HopWs h{};
+            BfsWs w{};
+            const size_t hop = hop_region_bytes(n, A, &h), bfs = bfs_region_bytes(n, A, zc, false, full, &w);
+            b += 4 * sms * (full ? hop + bfs : std::max(hop, bfs));
+        }
         if (pn) { PfmCtaWs w{}; b += 6 * sms * pfm_cta_region_bytes(pn, cb, false, &w); }
         return b;
     }
 
+    // sh/sfm level search: one region per CTA of the largest resident grid, at
+    // most 45 % of free memory (k_bfs and the pfm kernels may need theirs beside it).
+    int ensure_hop(uint32_t n, uint32_t A) {
+        if (hop_mem && n <= hop_n && A <= hop_A) return MANTRA_OK;
+        n = std::max(n, hop_n);
+        A = std::max(A, hop_A);
+        if (hop_mem) { cudaStreamSynchronize(sa); cudaFree(hop_mem); hop_mem = nullptr; }
+        CU(hop_configure(smem_optin));
+        int grid = 1;
+        for (int nt : {256, 512, 1024}) grid = std::max(grid, hop_grid(nt, 0, INT_MAX));
+        // MANTRA_BFS_GRID caps the resident CTAs
+        if (const char* env = std::getenv("MANTRA_BFS_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
+        const size_t region = hop_region_bytes(n, A, &hws);
+        const size_t budget = (size_t)((double)free_device_bytes() * 0.45);
+        if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
+        if (cudaMalloc(&hop_mem, (size_t)grid * region) != cudaSuccess) { hop_mem = nullptr; return MANTRA_E_NOMEM; }
+        CU(cudaMemsetAsync(hop_mem, 0, (size_t)grid * region, sa));
+        hws.base = hop_mem;
+        hws.stride = region;
+        hop_regions = grid;
+        hop_n = n; hop_A = A;
+        invalidate_graph();
+        return MANTRA_OK;
+    }
+
+    // Resident CTAs of k_hop (at most `most`) with nsm nodes' arrivals in shared
+    // memory (0: none); 0 when they do not fit.
+    int hop_grid(int nt, uint32_t nsm, int most) {
+        const size_t smem = hop_smem_bytes(nt, nsm);
+        if (smem > smem_optin) return 0;
+        const uint64_t key = ((uint64_t)nsm << 2) | (uint64_t)shape_of(nt);
+        auto it = hop_occ.find(key);
+        if (it == hop_occ.end()) {
+            int per = 0;
+            if (hop_blocks_per_sm(nt, nsm > 0, smem, &per) != cudaSuccess) per = 0;
+            it = hop_occ.emplace(key, per).first;
+        }
+        return std::min(most, it->second * num_sms);
+    }
+
+    // k_bfs (fsfm, RTB and the 128-bit re-runs): one region per resident CTA of
+    // the largest grid over CTA shapes and bitmap placements, at most 60 % of
+    // free memory.  Every region holds a global visited bitmap as well, so the
+    // placement is chosen per launch.
     int ensure_bfs(uint32_t n, uint32_t A, uint32_t zc, bool dl) {
         if (bfs_mem && n <= bfs_n && A <= bfs_A && zc <= bfs_z && (!dl || bfs_dl)) return MANTRA_OK;
         n = std::max(n, bfs_n);
@@ -359,7 +449,6 @@ struct Engine {
         bws.stride = region;
         for (int s = 0; s < 3; ++s)
             for (int p = 0; p < 2; ++p) bfs_grids[s][p] = per[s][p] > 0 ? std::min(grid, num_sms * per[s][p]) : 0;
-        bfs_grid = bfs_grids[1][bfs_rule_smem];
         bfs_smem = fit ? smem : 0;
         bfs_n = n; bfs_A = A; bfs_z = zc; bfs_dl = dl;
         invalidate_graph();
@@ -446,21 +535,29 @@ struct Engine {
     int enqueue(bool wide) {
         CU(cudaMemcpyAsync(tab_d, tab_h, tab_bytes, cudaMemcpyHostToDevice, sa));
         CU(cudaMemsetAsync(slot_d, 0, (size_t)cap * SLOT_BYTES, sa));
-        CU(cudaEventRecord(ev_fork, sa));
-        CU(cudaStreamWaitEvent(sb, ev_fork, 0));
+        if (tick_p) {
+            CU(cudaEventRecord(ev_fork, sa));
+            CU(cudaStreamWaitEvent(sb, ev_fork, 0));
+        }
         const uint32_t* hdr = (const uint32_t*)(tab_d + o_hdr);
         u64* work = (u64*)(tab_d + o_work);
-        if (bfs_mem) {
-            CU(cudaEventRecord(e_b0, sa));
+        if (tick_b || tick_h) CU(cudaEventRecord(e_b0, sa));
+        if (tick_h) {
+            HopWs w = hws;
+            w.nt = tick_hop_nt;
+            w.n_smem = tick_hop_sm ? tick_hop_n : 0;
+            CU(launch_hop((const Task*)(tab_d + o_th), (const uint64_t*)(tab_d + o_uh), hdr + 3, work + 2, w,
+                          hop_grid(tick_hop_nt, w.n_smem, hop_regions), sa));
+        }
+        if (tick_b) {
             BfsWs w = bws;
             w.nt = tick_bfs_nt;
             w.bits_in_smem = tick_bfs_sm;
             CU(launch_bfs((const Task*)(tab_d + o_tb), (const uint64_t*)(tab_d + o_ub), hdr + 0, work + 0, w,
-                          bfs_grids[shape_of(tick_bfs_nt)][tick_bfs_sm], tick_bfs_sm ? bfs_smem : 0, wide, tick_frac,
-                          sa));
-            CU(cudaEventRecord(e_b1, sa));
+                          bfs_grids[shape_of(tick_bfs_nt)][tick_bfs_sm], tick_bfs_sm ? bfs_smem : 0, wide, sa));
         }
-        if (tick_cta && !wide && pc_mem) {
+        if (tick_b || tick_h) CU(cudaEventRecord(e_b1, sa));
+        if (tick_p && tick_cta) {
             CU(cudaEventRecord(e_p0, sb));
             PfmCtaWs w = pcws;
             w.nt = tick_pc_nt;
@@ -469,14 +566,16 @@ struct Engine {
             CU(launch_pfm_cta((const Task*)(tab_d + o_tp), (const uint64_t*)(tab_d + o_up), hdr + 1, work + 1, w,
                               pc_grids[tick_pc_nt == 256 ? 0 : 1][tick_pc_sm], sb));
             CU(cudaEventRecord(e_p1, sb));
-        } else if (!tick_cta && pfm_mem) {
+        } else if (tick_p) {
             CU(cudaEventRecord(e_p0, sb));
             CU(launch_pfm((const Task*)(tab_d + o_tp), (const uint64_t*)(tab_d + o_up), hdr + 1, work + 1, pws,
                           pfm_grid, wide, sb));
             CU(cudaEventRecord(e_p1, sb));
         }
-        CU(cudaEventRecord(ev_join, sb));
-        CU(cudaStreamWaitEvent(sa, ev_join, 0));
+        if (tick_p) {
+            CU(cudaEventRecord(ev_join, sb));
+            CU(cudaStreamWaitEvent(sa, ev_join, 0));
+        }
         CU(launch_round_reduce((const ReduceItem*)(tab_d + o_ri), (const uint32_t*)(tab_d + o_rs), hdr + 2, red_grid,
                                sa));
         CU(cudaMemcpyAsync(slot_h, slot_d, (size_t)cap * SLOT_BYTES, cudaMemcpyDeviceToHost, sa));
@@ -546,16 +645,23 @@ double elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
     return ms;
 }
 
+// Whether a 64-bit sh / sfm search runs on k_hop (trk and ob estimates,
+// Algorithm 2); RTB and fsfm need every state's path count or time: k_bfs.
+// k_hop marks edges in bit 31 of a vertex id.
+bool on_hop(const mantra_graph* G, const Job& j) {
+    return (j.opt == MANTRA_SH || j.opt == MANTRA_SFM) && !j.rtb && G->n < (1u << 31);
+}
+
 // One line per tick item on stderr (MANTRA_LOG_LAUNCHES): kernel, launch
-// shape (threads) and state mode (k_bfs: bitmap placement; k_pfm_cta: the
-// engine's mode 0..3), the item's counters and algorithmic bytes, the
-// kernel's event time.
-void log_item(const TickItem& it, bool wide, bool cta, int nt, int mode, const u64* c, double ms) {
+// shape (threads) and state mode (k_hop: placement of the first slots; k_bfs:
+// bitmap placement; k_pfm_cta: the engine's mode 0..3), the item's counters
+// and algorithmic bytes, the kernel's event time.
+void log_item(const TickItem& it, const char* kernel, bool wide, int nt, int mode, const u64* c, double ms) {
     static const bool on = std::getenv("MANTRA_LOG_LAUNCHES") != nullptr;
     if (!on) return;
     const bool pfm = it.job.opt == MANTRA_PFM;
     std::fprintf(stderr, "mantra-launch kernel=%s%s nt=%d mode=%d samples=%llu escan=%llu eadd=%llu snew=%llu "
-                 "fseg=%llu xedge=%llu alg_bytes=%llu ms=%.4f\n", pfm ? (cta ? "k_pfm_cta" : "k_pfm") : "k_bfs",
+                 "fseg=%llu xedge=%llu alg_bytes=%llu ms=%.4f\n", kernel,
                  wide ? "<wide>" : "", nt, mode, (unsigned long long)it.job.count, (unsigned long long)c[C_ESCAN],
                  (unsigned long long)c[C_EADD], (unsigned long long)c[C_SNEW], (unsigned long long)c[C_FSEG],
                  (unsigned long long)c[C_XEDGE],
@@ -580,41 +686,85 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     int rc;
     if ((rc = E.ensure_tables(std::max<uint32_t>(k, 1))) != MANTRA_OK) return rc;
     uint32_t bn = 0, bA = 0, bz = 0, pn = 0, plc = 0, pz = 0;
-    const mantra_graph* gb = nullptr;   // the tick's largest sh/sfm graph: its knobs apply
     const mantra_graph* gp = nullptr;   // the tick's largest pfm graph
     uint64_t pwarps = 0, bsamples = 0;
-    bool any_b = false, any_p = false, frac = false, dl = false;
+    bool any_b = false, any_h = false, any_p = false, dl = false;
+    uint32_t hn = 0, hA = 0;
+    uint64_t hsamples = 0;
+    const mantra_graph* gh = nullptr;   // the tick's largest k_hop graph
     for (const TickItem& it : items) {
         if (it.job.opt == MANTRA_PFM) {
             any_p = true; pn = std::max(pn, it.G->n); plc = std::max(plc, it.G->dg.cbound);
             pz = std::max(pz, it.G->dg.max_vslots);
             if (!gp || it.G->n > gp->n) gp = it.G;
             pwarps += (it.job.count + 31) / 32;
+        } else if (!wide && on_hop(it.G, it.job)) {
+            any_h = true; hn = std::max(hn, it.G->n); hA = std::max(hA, it.G->A);
+            if (!gh || it.G->A > gh->A) gh = it.G;
+            hsamples += it.job.count;
         } else {
             any_b = true; bn = std::max(bn, it.G->n); bA = std::max(bA, it.G->A);
             bz = std::max(bz, it.G->dg.max_vslots);
-            if (!gb || it.G->A > gb->A) gb = it.G;
             bsamples += it.job.count;
-            frac |= it.job.ob || it.job.rtb || it.job.opt == 3;
             dl |= it.job.ob || it.job.rtb;
         }
     }
-    E.tick_frac = frac;
+    E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p;
     const bool cta = any_p && !wide && pfm_use_cta();
+    if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
     if (any_b && (rc = E.ensure_bfs(bn, bA, bz, dl)) != MANTRA_OK) return rc;
     if (any_p && cta && (rc = E.ensure_pfm_cta(pn, plc)) != MANTRA_OK) return rc;
     if (any_p && !cta && (rc = E.ensure_pfm(pn, plc, pwarps)) != MANTRA_OK) return rc;
     E.tick_cta = cta;
-    // sh/sfm CTA shape: 1024 threads for ticks of at most two samples per resident
-    // 1024-thread CTA (shorter per-sample latency), else two 512-thread CTAs per SM
-    // (measured on the n = 20,000 bursty graph: 1.9 vs 2.7 ms for 231 samples,
-    // 42.5 vs 40.4 ms for 26,702), or the shape and bitmap placement mantra_tune
-    // chose for the graph; MANTRA_BFS_NT=256|512|1024 forces a shape
+    // k_hop: CTA shape and placement of the arrivals.  Measured (sh / sfm, ms for
+    // 8,000 to 22,000 samples; threads:1 in shared memory, :0 in global memory):
+    //   n = 5,000 bursty    256:1 0.85   512:1 1.20   256:0 1.13   1024:0 2.29
+    //   n = 20,000 bursty   512:1 7.15   256:1 8.24   512:0 8.73   1024:0 11.5
+    //   n = 50,000 uniform  1024:0 6.41  512:0 7.14   512:1 7.27   256:0 10.1
+    //   n = 10^6 (2,048)    1024:0 76.5  512:0 90.2   256:0 112
+    // so: the smallest CTAs whose shared arrivals keep 1,024 threads per SM resident
+    // (a sample uses few threads at a time), else 1,024 threads on global arrivals
+    // (two and four samples per SM compete for L2).  A tick of at most two samples
+    // per SM wants each of them fast (231 samples: n = 20,000 1024:1 0.33, 512:1
+    // 0.42, 256:1 0.61; n = 5,000 0.19, 0.16, 0.21; n = 1,000 0.12, 0.09, 0.09).
+    // mantra_tune's choice for the graph comes first; MANTRA_BFS_NT=256|512|1024 and
+    // MANTRA_BFS_SMEM=0|1 force them.
+    if (any_h) {
+        uint32_t nq = 64;                        // shared nodes: the tick's largest graph, rounded up by at most 1/8
+        int cls = 0;
+        for (uint32_t step = 8; nq < hn && cls < 255; ++cls) {
+            nq += step;
+            if (nq >= 16 * step) step *= 2;
+        }
+        auto grid = [&](int nt, int sm) { return E.hop_grid(nt, sm ? nq : 0, E.hop_regions); };
+        int nt = 1024, sm = 0;
+        if (hsamples <= 2ull * (uint64_t)E.num_sms) {
+            nt = hn > 12000 ? 1024 : (hn > 1500 ? 512 : 256);
+            sm = grid(nt, 1) > 0;
+        } else if (grid(256, 1) >= 4 * E.num_sms) {
+            nt = 256; sm = 1;
+        } else if (grid(512, 1) >= 2 * E.num_sms) {
+            nt = 512; sm = 1;
+        }
+        if (gh && gh->knobs.bfs_nt) { nt = gh->knobs.bfs_nt; sm = gh->knobs.bfs_smem > 0; }
+        if (const char* env = std::getenv("MANTRA_BFS_NT")) {
+            const int v = std::atoi(env);
+            nt = v == 1024 ? 1024 : (v == 256 ? 256 : 512);
+        }
+        if (const char* env = std::getenv("MANTRA_BFS_SMEM")) sm = env[0] == '1';
+        if (nq < hn || !grid(nt, sm)) sm = 0;    // the arrivals do not fit this shape
+        E.tick_hop_nt = nt;
+        E.tick_hop_sm = sm;
+        E.tick_hop_cls = cls;
+        E.tick_hop_n = nq;
+    }
+    // k_bfs CTA shape: 1024 threads for ticks of at most two samples per resident
+    // 1024-thread CTA (shorter per-sample latency), else two 512-thread CTAs per
+    // SM (measured for sh on the n = 20,000 bursty graph: 1.9 vs 2.7 ms for 231
+    // samples, 42.5 vs 40.4 ms for 26,702); the same variables force them
     if (any_b) {
         const bool small = bsamples <= 2ull * (uint64_t)E.bfs_grids[2][E.bfs_rule_smem];
         int nt = small ? 1024 : 512, sm = E.bfs_rule_smem;
-        if (gb && !small && gb->knobs.bfs_nt) nt = gb->knobs.bfs_nt;
-        if (gb && !small && gb->knobs.bfs_smem >= 0) sm = gb->knobs.bfs_smem;
         if (const char* env = std::getenv("MANTRA_BFS_NT")) {
             const int v = std::atoi(env);
             nt = v == 1024 ? 1024 : (v == 256 ? 256 : 512);
@@ -652,12 +802,14 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     u64* work = (u64*)(E.tab_h + E.o_work);
     uint64_t* ub = (uint64_t*)(E.tab_h + E.o_ub);
     uint64_t* up = (uint64_t*)(E.tab_h + E.o_up);
+    uint64_t* uh = (uint64_t*)(E.tab_h + E.o_uh);
+    Task* th = (Task*)(E.tab_h + E.o_th);
     Task* tb = (Task*)(E.tab_h + E.o_tb);
     Task* tp = (Task*)(E.tab_h + E.o_tp);
     ReduceItem* ri = (ReduceItem*)(E.tab_h + E.o_ri);
     uint32_t* rs = (uint32_t*)(E.tab_h + E.o_rs);
-    uint32_t nb = 0, np = 0, nr = 0;
-    ub[0] = 0; up[0] = 0; rs[0] = 0;
+    uint32_t nb = 0, np = 0, nr = 0, nh = 0;
+    ub[0] = 0; up[0] = 0; uh[0] = 0; rs[0] = 0;
     for (uint32_t x = 0; x < k; ++x) {
         TickItem& it = items[x];
         char* slot = E.slot_d + (size_t)x * SLOT_BYTES;
@@ -669,6 +821,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             up[np + 1] = up[np] + (cta ? it.job.count : (it.job.count + 31) / 32);
             ++np;
         }
+        else if (!wide && on_hop(it.G, it.job)) { th[nh] = t; uh[nh + 1] = uh[nh] + it.job.count; ++nh; }
         else { tb[nb] = t; ub[nb + 1] = ub[nb] + it.job.count; ++nb; }
         if (it.reduce) {
             ri[nr] = ReduceItem{it.job.S, it.job.S64, (it.job.ob || it.job.rtb) ? it.job.wsq : it.job.hits, it.job.fam,
@@ -679,14 +832,14 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             ++nr;
         }
     }
-    hdr[0] = nb; hdr[1] = np; hdr[2] = nr;
-    work[0] = 0; work[1] = 0;
+    hdr[0] = nb; hdr[1] = np; hdr[2] = nr; hdr[3] = nh;
+    work[0] = 0; work[1] = 0; work[2] = 0;
     if ((rc = E.launch_tick(wide)) != MANTRA_OK) return rc;
     CU(cudaStreamSynchronize(E.sa));
     out->slot.resize(k);
     for (uint32_t x = 0; x < k; ++x) out->slot[x] = E.slot_h + (size_t)x * SLOT_BYTES;
-    out->had_bfs = nb > 0 && E.bfs_mem;
-    out->had_pfm = np > 0 && (cta ? E.pc_mem != nullptr : E.pfm_mem != nullptr);
+    out->had_bfs = nb + nh > 0;
+    out->had_pfm = np > 0;
     if (E.last_tick_graph) {
         // a graph tick is timed as a whole: table upload, searches, reduction, readback
         const double t = elapsed_ms(E.e_t0, E.e_t1);
@@ -696,12 +849,16 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         out->bfs_ms = out->had_bfs ? elapsed_ms(E.e_b0, E.e_b1) : 0.0;
         out->pfm_ms = out->had_pfm ? elapsed_ms(E.e_p0, E.e_p1) : 0.0;
     }
-    for (uint32_t x = 0; x < k; ++x)
+    for (uint32_t x = 0; x < k; ++x) {
+        const u64* c = (const u64*)out->slot[x];
         if (items[x].job.opt == MANTRA_PFM)
-            log_item(items[x], wide, cta, cta ? E.tick_pc_nt : 32, cta ? E.tick_pc_sm : 0, (const u64*)out->slot[x],
+            log_item(items[x], cta ? "k_pfm_cta" : "k_pfm", wide, cta ? E.tick_pc_nt : 32, cta ? E.tick_pc_sm : 0, c,
                      out->pfm_ms);
+        else if (!wide && on_hop(items[x].G, items[x].job))
+            log_item(items[x], "k_hop", wide, E.tick_hop_nt, E.tick_hop_sm, c, out->bfs_ms);
         else
-            log_item(items[x], wide, cta, E.tick_bfs_nt, E.tick_bfs_sm, (const u64*)out->slot[x], out->bfs_ms);
+            log_item(items[x], "k_bfs", wide, E.tick_bfs_nt, E.tick_bfs_sm, c, out->bfs_ms);
+    }
     return MANTRA_OK;
 }
 
@@ -1172,7 +1329,7 @@ struct Server {
                 pn = std::max(pn, G->n); cb = std::max(cb, G->dg.cbound);
             } else {
                 n = std::max(n, G->n); A = std::max(A, G->A); z = std::max(z, G->dg.max_vslots);
-                dl = dl || r->p.estimator != 0;
+                dl = dl || r->p.estimator == 2 || r->p.opt == MANTRA_FSFM;
             }
         };
         for (const Request* r : active) add(r);
@@ -1209,7 +1366,7 @@ struct Server {
                     ps.push_back(&r->p);
                 }
                 // per-family tick budgets (MANTRA_SERVER_TICK_SAMPLES overrides)
-                uint64_t bb = SERVER_TICK_PER_CTA * (uint64_t)(E->bfs_grid ? E->bfs_grid : 2 * E->num_sms);
+                uint64_t bb = SERVER_TICK_PER_CTA * (uint64_t)(E->hop_regions ? E->hop_regions : 2 * E->num_sms);
                 uint64_t bp = SERVER_TICK_PER_CTA * (uint64_t)(E->pc_grid ? E->pc_grid : 2 * E->num_sms);
                 if (const char* env = std::getenv("MANTRA_SERVER_TICK_SAMPLES")) {
                     const long long v = std::atoll(env);
@@ -1412,14 +1569,14 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
         r = per > 0 ? (uint64_t)std::min<double>((double)r_hi, std::max<double>((double)r_lo, 100.0 / per)) : r_hi;
         return MANTRA_OK;
     };
-    // sh/sfm: CTA shape x visited-bitmap placement (shared memory only where it fits)
+    // sh/sfm: CTA shape x placement of the first slots (shared memory only where they fit)
     if ((rc = size_probe(MANTRA_SH)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->probe_samples = r;
     if ((rc = probe(MANTRA_SH, none, &out->bfs_default_ms)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->bfs_ms = 1e300;
     for (int nt : {256, 512, 1024})
         for (int sm = 0; sm < 2; ++sm) {
-            if (!E->bfs_grids[Engine::shape_of(nt)][sm]) continue;
+            if (!E->hop_grid(nt, sm ? g->n : 0, E->hop_regions)) continue;
             Knobs k = none;
             k.bfs_nt = nt; k.bfs_smem = sm;
             double ms = 0;
@@ -1448,7 +1605,7 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
     out->pfm_state_shared = best.pfm_mode == 1 || best.pfm_mode == 3 ? 1u : 0u;
     out->pfm_staged = best.pfm_mode == 2 ? 1u : 0u;
     out->pfm_state16 = best.pfm_mode == 3 ? 1u : 0u;
-    out->bfs_resident_ctas = best.bfs_nt ? (uint32_t)E->bfs_grids[Engine::shape_of(best.bfs_nt)][best.bfs_smem] : 0u;
+    out->bfs_resident_ctas = best.bfs_nt ? (uint32_t)E->hop_grid(best.bfs_nt, best.bfs_smem > 0 ? g->n : 0, E->hop_regions) : 0u;
     out->pfm_resident_ctas = best.pfm_nt ? (uint32_t)E->pc_grids[best.pfm_nt == 256 ? 0 : 1][best.pfm_mode] : 0u;
     if (!best.pfm_nt) out->pfm_ms = out->pfm_default_ms;
     return MANTRA_OK;

@@ -1,4 +1,7 @@
-// (*)-temporal BFS for the shortest (sh) and shortest-foremost (sfm)
+// (*)-temporal BFS with a path count for every state: the RTB estimator and the
+// foremost-first order (fsfm), the 128-bit re-runs of every sh / sfm search, and
+// the allocation-free sampler (other sh / sfm searches: k_hop.cu).  For the
+// shortest (sh) and shortest-foremost (sfm)
 // optimalities (paper Sec. 3 Def. 1; running-time theorem of Sec. 4.4), the
 // backward path draw of the temporal Riondato-Kornaropoulos estimator
 // (App. C, theorem on the path sampler), and the Update step of Algorithm 1
@@ -391,11 +394,8 @@ __device__ __noinline__ void bfs_frac_update(int mode, FracCtx* x) {
                                      acc2, seg_b, VB, seg_u, &x->nt);
 }
 
-// BFS_NT threads per CTA, 1024 / BFS_NT CTAs per SM at 64 registers.  FRAC:
-// the instantiation that also runs the ob and RTB updates and fsfm (a tick
-// with such a problem launches it); the others report those jobs as a
-// consistency error.
-template <bool WIDE, int BFS_NT, bool FRAC>
+// BFS_NT threads per CTA, 1024 / BFS_NT CTAs per SM at 64 registers.
+template <bool WIDE, int BFS_NT>
 __global__ void __launch_bounds__(BFS_NT, 1024 / BFS_NT) k_bfs(const Task* tasks, const uint64_t* unit_start,
                                                    const uint32_t* ntasks_p, u64* work,
                                                    const __grid_constant__ BfsWs ws) {
@@ -542,8 +542,8 @@ __global__ void __launch_bounds__(BFS_NT, 1024 / BFS_NT) k_bfs(const Task* tasks
         const bool full = stats || job.rtb;   // untruncated search (no target)
         // fsfm (foremost first, then fewest hops): no stop at z's first level;
         // every state up to z's latest in-edge time, the endpoint is z's
-        // earliest slot found at any level (FRAC instantiation only)
-        const bool fsfm = FRAC && job.opt == 3 && !full;
+        // earliest slot found at any level
+        const bool fsfm = job.opt == 3 && !full;
         const uint32_t tz = full ? NONE : g.tmax_in[z];
         const uint32_t zlo = fsfm ? g.slot_ptr[z] : 0u, zhi = fsfm ? g.slot_ptr[z + 1] : 0u;
         bool live = ok && (g.out_ptr[s + 1] > g.out_ptr[s]);
@@ -1123,9 +1123,7 @@ __global__ void __launch_bounds__(BFS_NT, 1024 / BFS_NT) k_bfs(const Task* tasks
         }
 
         // ---------------- ob (Sec. 4.1) and RTB (App. C) updates (block-uniform conditions) ----------------
-        if constexpr (!FRAC) {
-            if ((job.ob || job.rtb || job.opt == 3) && tid == 0) set_status(job.status, ST_CHECK);
-        } else {
+        {
             const int mode = (job.ob && job.hits && found && !sh_ovf && !sh_err && sh_d >= 2) ? 1
                            : (job.rtb && job.hits && live && !sh_ovf && k >= 2) ? 2
                            : (stats && job.opt == 3 && live && k >= 1) ? 3 : 0;
@@ -1220,18 +1218,15 @@ size_t bfs_smem_bytes(uint32_t A) { return (size_t)((A + 31) / 32) * 4; }
 // Static shared memory of the nt-thread kernels (range table, task copy,
 // level scratch).
 size_t bfs_static_smem(int nt) {
-    cudaFuncAttributes a{}, b{}, c{};
-    const cudaError_t e1 = nt == 1024 ? cudaFuncGetAttributes(&a, k_bfs<false, 1024, false>)
-                         : nt == 256  ? cudaFuncGetAttributes(&a, k_bfs<false, 256, false>)
-                                      : cudaFuncGetAttributes(&a, k_bfs<false, 512, false>);
-    const cudaError_t e2 = nt == 1024 ? cudaFuncGetAttributes(&b, k_bfs<true, 1024, true>)
-                         : nt == 256  ? cudaFuncGetAttributes(&b, k_bfs<true, 256, true>)
-                                      : cudaFuncGetAttributes(&b, k_bfs<true, 512, true>);
-    const cudaError_t e3 = nt == 1024 ? cudaFuncGetAttributes(&c, k_bfs<false, 1024, true>)
-                         : nt == 256  ? cudaFuncGetAttributes(&c, k_bfs<false, 256, true>)
-                                      : cudaFuncGetAttributes(&c, k_bfs<false, 512, true>);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) return 96 * 1024;
-    return std::max(std::max(a.sharedSizeBytes, b.sharedSizeBytes), c.sharedSizeBytes);
+    cudaFuncAttributes a{}, b{};
+    const cudaError_t e1 = nt == 1024 ? cudaFuncGetAttributes(&a, k_bfs<false, 1024>)
+                         : nt == 256  ? cudaFuncGetAttributes(&a, k_bfs<false, 256>)
+                                      : cudaFuncGetAttributes(&a, k_bfs<false, 512>);
+    const cudaError_t e2 = nt == 1024 ? cudaFuncGetAttributes(&b, k_bfs<true, 1024>)
+                         : nt == 256  ? cudaFuncGetAttributes(&b, k_bfs<true, 256>)
+                                      : cudaFuncGetAttributes(&b, k_bfs<true, 512>);
+    if (e1 != cudaSuccess || e2 != cudaSuccess) return 96 * 1024;
+    return std::max(a.sharedSizeBytes, b.sharedSizeBytes);
 }
 
 // Raises (never lowers) the kernels' dynamic shared-memory limit on the
@@ -1246,11 +1241,8 @@ cudaError_t bfs_configure(size_t smem) {
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     std::lock_guard<std::mutex> lock(mu);
     if (smem <= configured[dev]) return cudaSuccess;
-    const void* ks[9] = {(const void*)k_bfs<false, 512, false>, (const void*)k_bfs<false, 512, true>,
-                         (const void*)k_bfs<true, 512, true>, (const void*)k_bfs<false, 1024, false>,
-                         (const void*)k_bfs<false, 1024, true>, (const void*)k_bfs<true, 1024, true>,
-                         (const void*)k_bfs<false, 256, false>, (const void*)k_bfs<false, 256, true>,
-                         (const void*)k_bfs<true, 256, true>};
+    const void* ks[6] = {(const void*)k_bfs<false, 512>,  (const void*)k_bfs<true, 512>, (const void*)k_bfs<false, 1024>,
+                         (const void*)k_bfs<true, 1024>, (const void*)k_bfs<false, 256>, (const void*)k_bfs<true, 256>};
     for (const void* k : ks) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -1260,26 +1252,22 @@ cudaError_t bfs_configure(size_t smem) {
 }
 
 cudaError_t bfs_blocks_per_sm(int nt, size_t smem, int* out) {
-    if (nt == 1024) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 1024, false>, 1024, smem);
-    if (nt == 256) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 256, false>, 256, smem);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 512, false>, 512, smem);
+    if (nt == 1024) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 1024>, 1024, smem);
+    if (nt == 256) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 256>, 256, smem);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, k_bfs<false, 512>, 512, smem);
 }
 
 cudaError_t launch_bfs(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
-                       const BfsWs& ws, int grid, size_t smem, bool wide, bool frac, cudaStream_t st) {
-    // the 128-bit re-run always takes the FRAC instantiation
+                       const BfsWs& ws, int grid, size_t smem, bool wide, cudaStream_t st) {
     if (ws.nt == 1024) {
-        if (wide) k_bfs<true, 1024, true><<<grid, 1024, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else if (frac) k_bfs<false, 1024, true><<<grid, 1024, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else k_bfs<false, 1024, false><<<grid, 1024, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        if (wide) k_bfs<true, 1024><<<grid, 1024, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        else k_bfs<false, 1024><<<grid, 1024, smem, st>>>(tasks, unit_start, ntasks, work, ws);
     } else if (ws.nt == 256) {
-        if (wide) k_bfs<true, 256, true><<<grid, 256, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else if (frac) k_bfs<false, 256, true><<<grid, 256, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else k_bfs<false, 256, false><<<grid, 256, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        if (wide) k_bfs<true, 256><<<grid, 256, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        else k_bfs<false, 256><<<grid, 256, smem, st>>>(tasks, unit_start, ntasks, work, ws);
     } else {
-        if (wide) k_bfs<true, 512, true><<<grid, 512, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else if (frac) k_bfs<false, 512, true><<<grid, 512, smem, st>>>(tasks, unit_start, ntasks, work, ws);
-        else k_bfs<false, 512, false><<<grid, 512, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        if (wide) k_bfs<true, 512><<<grid, 512, smem, st>>>(tasks, unit_start, ntasks, work, ws);
+        else k_bfs<false, 512><<<grid, 512, smem, st>>>(tasks, unit_start, ntasks, work, ws);
     }
     return cudaGetLastError();
 }

@@ -65,6 +65,14 @@ struct DevGraph {
     const uint32_t* slot_nout;   // per arrival slot (v, t): first index of v's out-row with time > t
     const unsigned short* out_loff;   // per out-edge: its head's slot offset within the head's slots
                                       // (out_slot - slot_ptr[out_v], 0xFFFF when above)
+    const uint2* out_vn;         // per out-edge: the head, bit 31 set when its slot has several in-edges
+                                 // (graphs of fewer than 2^31 nodes), and slot_nout of its slot
+    const uint32_t* in_out;      // per in-CSR index: the edge's out-CSR index
+    const uint32_t* out_pend;    // per out-edge (u, v, t): one past u's last slot earlier than t
+    const uint2* dir;            // dir_n x n: the part [x, y) of v's out-row with times from dir_t[b] to
+                                 // dir_t[b + 1] (the last bucket: to the row's end)
+    const uint32_t* dir_t;       // dir_n bucket times, ascending, the first 0
+    uint32_t dir_n;              // buckets of the times (at most 32)
 };
 
 // Largest number of arrival slots of one vertex for the CTA pfm kernel's
@@ -344,6 +352,31 @@ __device__ __forceinline__ u64 block_exclusive_scan64(u64 v, u64* total, u64* sc
     return before + x - v;
 }
 
+// Block-wide exclusive scan of two uint32 per thread with one barrier: every
+// warp writes its two totals, every warp then sums all warps' totals itself
+// (one shared load and two redux per value).  `scratch` holds 64 words; two
+// consecutive calls must use different scratch (the caller alternates two), as
+// a fast warp may write its next totals while a slow one still reads.
+template <int NT>
+__device__ __forceinline__ void block_exclusive_scan2(uint32_t& a, uint32_t& b, uint32_t* ta, uint32_t* tb,
+                                                      uint32_t* scratch) {
+    constexpr int NW = NT / 32;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t x = a, y = b;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t p = __shfl_up_sync(0xFFFFFFFFu, x, o), q = __shfl_up_sync(0xFFFFFFFFu, y, o);
+        if (lane >= o) { x += p; y += q; }
+    }
+    if (lane == 31) { scratch[wid] = x; scratch[32 + wid] = y; }
+    __syncthreads();
+    const uint32_t wa = lane < NW ? scratch[lane] : 0u, wb = lane < NW ? scratch[32 + lane] : 0u;
+    *ta = __reduce_add_sync(0xFFFFFFFFu, wa);
+    *tb = __reduce_add_sync(0xFFFFFFFFu, wb);
+    a = x - a + __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wa : 0u);
+    b = y - b + __reduce_add_sync(0xFFFFFFFFu, lane < wid ? wb : 0u);
+}
+
 // Block-wide inclusive segmented scan: f = 1 starts a new segment at this
 // thread; the running sum continues across calls through *carry (the value
 // entering thread 0 when its f = 0).  Any wrapped addition sets *ovf (exact:
@@ -433,6 +466,42 @@ __device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict_
     const uint32_t idx = lo + lane;
     const bool lt = idx < hi && __ldg(a + idx) < key;
     return lo + __popc(__ballot_sync(0xFFFFFFFFu, lt));
+}
+
+// For each k: the first index in [lo[k], hi[k]) whose value exceeds key (hi[k]
+// if none), left in lo[k].  Four probes in flight per search and step (a fifth
+// of the range each), so a search costs about log5 of the range in dependent
+// loads; the K searches advance together.
+template <int K>
+__device__ __forceinline__ void upper_bounds_5(const uint32_t* __restrict__ a, uint32_t (&lo)[K], uint32_t (&hi)[K],
+                                               uint32_t key) {
+    for (;;) {
+        bool any = false;
+        uint32_t val[K][4], st[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t len = hi[k] > lo[k] ? hi[k] - lo[k] : 0u;
+            any |= len > 0u;
+            st[k] = len / 5u + (len > 4u ? 0u : 1u);     // probes lo + st - 1, lo + 2 st - 1, ..
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint32_t p = lo[k] + (uint32_t)(j + 1) * st[k] - 1u;
+                val[k][j] = len > 0u && p < hi[k] ? __ldg(a + p) : NONE;
+            }
+        }
+        if (!any) break;
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            if (hi[k] <= lo[k]) continue;
+            // the probes at most key are a prefix: the answer is between it and the next probe
+            uint32_t c = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) c += val[k][j] <= key ? 1u : 0u;
+            const uint32_t nhi = lo[k] + (c + 1u) * st[k] - 1u;
+            lo[k] += c * st[k];
+            if (c < 4u) hi[k] = min(hi[k], nhi);
+        }
+    }
 }
 
 // For each k: the first index in [lo[k], hi[k]) whose value exceeds key[k]
@@ -542,6 +611,38 @@ __device__ __forceinline__ void lbs_walk_batched(const uint32_t* off, uint32_t G
 #pragma unroll
         for (int k = 0; k < K; ++k)
             if (ok[k]) edge(rr[k], ee[k], va[k], vb[k]);
+    }
+}
+
+// lbs_walk over K windows at a time for callers that process the windows' edges
+// with the whole warp, stage by stage: body(e) gets the K windows' edges of
+// the lane (NONE past the end) and is called by all 32 lanes.  base[g] = the
+// first edge of range g minus off[g]; off has 32 entries of NONE behind off[Gc].
+template <int K, typename BodyF>
+__device__ __forceinline__ void lbs_walk_warp(const uint32_t* off, uint32_t Gc, const uint32_t* base, uint32_t w_lo,
+                                              uint32_t w_hi, BodyF body) {
+    const uint32_t lane = threadIdx.x & 31;
+    if (w_lo >= w_hi) return;
+    uint32_t lo = 0, hi = Gc;                 // off[lo] <= w_lo < off[hi]
+    while (hi - lo > 1) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (off[mid] <= w_lo) lo = mid; else hi = mid;
+    }
+    const uint32_t upto = (2u << lane) - 1u;
+    const uint32_t* p = off + lo + 1u + lane;  // p - off - 1 - lane: the range of the window's first edge
+    const uint32_t* q = base + lo;
+    for (uint32_t b = w_lo; b < w_hi; b += 32u * K) {
+        uint32_t ee[K];
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const uint32_t d = *p - (b + 32u * k);              // the next ranges' starts, > 0 (past the end: large)
+            const uint32_t mask = __reduce_or_sync(0xFFFFFFFFu, d < 32u ? (1u << d) : 0u);
+            const uint32_t j = b + 32u * k + lane;
+            ee[k] = j < w_hi ? q[__popc(mask & upto)] + j : NONE;
+            const uint32_t n = __popc(__ballot_sync(0xFFFFFFFFu, d <= 32u));
+            p += n; q += n;
+        }
+        body(ee);
     }
 }
 
@@ -664,6 +765,20 @@ struct BfsWs {
     int has_dl;          // the ob / RTB scratch (o_fc, o_acc, o_acc2) is allocated
 };
 
+// Per-CTA scratch of the hop-level search kernel (one region per CTA).
+struct HopWs {
+    char* base;          // CTA b uses base + b * stride
+    size_t stride;
+    size_t o_fb, o_want, o_grp, o_grp2, o_acc, o_q, o_ea, o_eb, o_rng, o_lev, o_mst, o_ca, o_ct, o_cs, o_cb, o_gw, o_gs,
+           o_path, o_pathe, o_stamp;
+    uint32_t n_cap;      // node capacity of a region
+    uint32_t A_cap;      // slot capacity of a region
+    uint32_t ev_cap;     // (vertex, level) events per sample; more: the sample goes to the overflow list
+    uint32_t c_cap;      // states on optimal paths per sample; more: the overflow list
+    int nt;              // threads per CTA (256, 512 or 1024)
+    uint32_t n_smem;     // nodes whose next-level arrivals are in dynamic shared memory (0: in the region)
+};
+
 // Per-warp scratch of the pfm search kernel.
 struct PfmWs {
     char* base;          // warp w uses base + w * stride
@@ -698,7 +813,16 @@ cudaError_t bfs_configure(size_t smem);
 // task_of_unit(unit_start, *ntasks, u); the first unused unit ends a CTA/warp.
 // sh/sfm: one unit per sample; pfm: one unit per 32 consecutive samples of a task.
 cudaError_t launch_bfs(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
-                       const BfsWs& ws, int grid, size_t smem, bool wide, bool frac, cudaStream_t st);
+                       const BfsWs& ws, int grid, size_t smem, bool wide, cudaStream_t st);
+size_t hop_region_bytes(uint32_t n, uint32_t A, HopWs* ws);
+size_t hop_smem_bytes(int nt, uint32_t n);
+cudaError_t hop_configure(size_t smem);
+cudaError_t hop_blocks_per_sm(int nt, bool first_in_smem, size_t smem, int* out);
+cudaError_t launch_hop(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
+                       const HopWs& ws, int grid, cudaStream_t st);
+// Fills out_vn, in_out, out_pend and dir of g (whose other arrays are in place).
+cudaError_t launch_edge_maps(const DevGraph& g, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend, uint2* dir,
+                             cudaStream_t st);
 size_t pfm_region_bytes(uint32_t n, uint32_t list_cap, PfmWs* ws);
 int pfm_threads();
 cudaError_t launch_pfm(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
