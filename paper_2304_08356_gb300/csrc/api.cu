@@ -46,6 +46,8 @@ struct mantra_graph {
     uint64_t self_loops = 0, duplicates = 0;
     DevGraph dg{};
     void* dmem = nullptr;
+    void* wmem = nullptr;   // waves of the stream (k_sweep), or none
+    size_t b_dmem = 0, b_wmem = 0;
     int device = 0;
     Knobs knobs;         // set by mantra_tune
 };
@@ -63,70 +65,6 @@ int cuda_fail(cudaError_t e, const char* what, int line) {
 
 size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// ---------------------------------------------------------------------------
-// Temporal-edge store (paper Sec. 3: the temporal graph; the paper's own code
-// keeps a sparse n x |T| table, here every arrival appearance (v,t) gets a
-// dense slot id).  The host team of store.cu builds the arrays; this uploads
-// them into one device allocation, each array from its page-locked buffer.
-// ---------------------------------------------------------------------------
-int upload_store(const StoreHost& H, mantra_graph* G, cudaStream_t st) {
-    const uint32_t** dst[SA_COUNT] = {};
-    dst[SA_OUT_PTR] = &G->dg.out_ptr;   dst[SA_OUT_V] = &G->dg.out_v;       dst[SA_OUT_T] = &G->dg.out_t;
-    dst[SA_OUT_SLOT] = &G->dg.out_slot; dst[SA_SLOT_PTR] = &G->dg.slot_ptr; dst[SA_SLOT_T] = &G->dg.slot_t;
-    dst[SA_SLOT_V] = &G->dg.slot_v;     dst[SA_SLOT_IN] = &G->dg.slot_in;   dst[SA_IN_U] = &G->dg.in_u;
-    dst[SA_IN_SLOT] = &G->dg.in_slot;   dst[SA_ST_U] = &G->dg.st_u;         dst[SA_ST_V] = &G->dg.st_v;
-    dst[SA_ST_T] = &G->dg.st_t;         dst[SA_TMAX_IN] = &G->dg.tmax_in;   dst[SA_TMIN_OUT] = &G->dg.tmin_out;
-    dst[SA_IN_UEDGE] = &G->dg.in_uedge; dst[SA_SLOT_NOUT] = &G->dg.slot_nout;
-    const uint32_t* loff_words = nullptr;   // 16-bit entries, two per word
-    dst[SA_OUT_LOFF] = &loff_words;
-    size_t total = 0;
-    for (int k = 0; k < SA_COUNT; ++k) total += al256((H.len[k] + 1) * 4);
-    // filled on the device: the edges' head and continuation, the in-edges' out-CSR
-    // index, the edges' usable slots, and the out-rows cut at up to 32 times (as many as the mean row has
-    // edges, so that the directory is no larger than the edge arrays)
-    uint32_t nb = 1;
-    while (nb < 32 && (uint64_t)nb * H.n < H.m) nb *= 2;
-    const size_t o_vn = total;
-    total += al256(((size_t)H.m + 1) * 8);
-    const size_t o_io = total;
-    total += al256(((size_t)H.m + 1) * 4);
-    const size_t o_pe = total;
-    total += al256(((size_t)H.m + 1) * 4);
-    const size_t o_dir = total;
-    total += al256((size_t)nb * H.n * 8);
-    const size_t o_dt = total;
-    total += al256(32 * 4);
-    if (cudaMalloc(&G->dmem, total) != cudaSuccess) return MANTRA_E_NOMEM;
-    size_t off = 0;
-    for (int k = 0; k < SA_COUNT; ++k) {
-        char* p = (char*)G->dmem + off;
-        if (H.len[k]) CU(cudaMemcpyAsync(p, H.arr[k], H.len[k] * 4, cudaMemcpyHostToDevice, st));
-        *dst[k] = (const uint32_t*)p;
-        off += al256((H.len[k] + 1) * 4);
-    }
-    uint32_t dt[32] = {};
-    for (uint32_t j = 1; j < nb; ++j) dt[j] = H.arr[SA_ST_T][(size_t)j * H.m / nb];   // m > n here
-    char* base = (char*)G->dmem;
-    CU(cudaMemcpyAsync(base + o_dt, dt, sizeof dt, cudaMemcpyHostToDevice, st));
-    G->dg.n = H.n; G->dg.m = H.m; G->dg.A = H.A;
-    G->dg.out_vn = (const uint2*)(base + o_vn);
-    G->dg.in_out = (const uint32_t*)(base + o_io);
-    G->dg.out_pend = (const uint32_t*)(base + o_pe);
-    G->dg.dir = (const uint2*)(base + o_dir);
-    G->dg.dir_t = (const uint32_t*)(base + o_dt);
-    G->dg.dir_n = nb;
-    CU(launch_edge_maps(G->dg, (uint2*)(base + o_vn), (uint32_t*)(base + o_io), (uint32_t*)(base + o_pe),
-                        (uint2*)(base + o_dir), st));
-    CU(cudaStreamSynchronize(st));
-    G->dg.out_loff = reinterpret_cast<const unsigned short*>(loff_words);
-    G->n = H.n; G->m = H.m; G->A = H.A; G->n_uedge = H.n_uedge;
-    G->self_loops = H.self_loops; G->duplicates = H.duplicates;
-    G->dg.n = H.n; G->dg.A = H.A; G->dg.m = H.m; G->dg.n_uedge = H.n_uedge;
-    G->dg.cbound = H.cbound; G->dg.max_slot_in = H.max_slot_in; G->dg.max_vslots = H.max_vslots;
-    return MANTRA_OK;
-}
-
-
 size_t free_device_bytes() {
     size_t fr = 0, tot = 0;
     if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) return 0;
@@ -139,7 +77,7 @@ double now_s() {
 
 // ---------------------------------------------------------------------------
 // Device memory pool: blocks kept by exact (256-rounded) size and reused by
-// later problems; at most kPoolCacheBytes stay cached.
+// later problems and graphs; at most kPoolCacheBytes stay cached.
 // ---------------------------------------------------------------------------
 constexpr size_t kPoolCacheBytes = (size_t)8 << 30;
 
@@ -175,6 +113,105 @@ struct DevPool {
         cached = 0;
     }
 };
+
+// ---------------------------------------------------------------------------
+// Temporal-edge store (paper Sec. 3: the temporal graph; the paper's own code
+// keeps a sparse n x |T| table, here every arrival appearance (v,t) gets a
+// dense slot id).  The host team of store.cu builds the arrays; this uploads
+// them into one device allocation, each array from its page-locked buffer.
+// ---------------------------------------------------------------------------
+int upload_store(const StoreHost& H, mantra_graph* G, DevPool& pool, cudaStream_t st) {
+    const uint32_t** dst[SA_COUNT] = {};
+    dst[SA_OUT_PTR] = &G->dg.out_ptr;   dst[SA_OUT_V] = &G->dg.out_v;       dst[SA_OUT_T] = &G->dg.out_t;
+    dst[SA_OUT_SLOT] = &G->dg.out_slot; dst[SA_SLOT_PTR] = &G->dg.slot_ptr; dst[SA_SLOT_T] = &G->dg.slot_t;
+    dst[SA_SLOT_V] = &G->dg.slot_v;     dst[SA_SLOT_IN] = &G->dg.slot_in;   dst[SA_IN_U] = &G->dg.in_u;
+    dst[SA_IN_SLOT] = &G->dg.in_slot;   dst[SA_ST_U] = &G->dg.st_u;         dst[SA_ST_V] = &G->dg.st_v;
+    dst[SA_ST_T] = &G->dg.st_t;         dst[SA_TMAX_IN] = &G->dg.tmax_in;   dst[SA_TMIN_OUT] = &G->dg.tmin_out;
+    dst[SA_IN_UEDGE] = &G->dg.in_uedge; dst[SA_SLOT_NOUT] = &G->dg.slot_nout;
+    const uint32_t* loff_words = nullptr;   // 16-bit entries, two per word
+    dst[SA_OUT_LOFF] = &loff_words;
+    size_t total = 0;
+    for (int k = 0; k < SA_COUNT; ++k) total += al256((H.len[k] + 1) * 4);
+    // filled on the device: the edges' head and continuation, the in-edges' out-CSR
+    // index, the edges' usable slots, and the out-rows cut at up to 32 times (as many as the mean row has
+    // edges, so that the directory is no larger than the edge arrays)
+    uint32_t nb = 1;
+    while (nb < 32 && (uint64_t)nb * H.n < H.m) nb *= 2;
+    const size_t o_vn = total;
+    total += al256(((size_t)H.m + 1) * 8);
+    const size_t o_io = total;
+    total += al256(((size_t)H.m + 1) * 4);
+    const size_t o_pe = total;
+    total += al256(((size_t)H.m + 1) * 4);
+    const size_t o_dir = total;
+    total += al256((size_t)nb * H.n * 8);
+    const size_t o_dt = total;
+    total += al256(32 * 4);
+    G->dmem = pool.get(total);
+    if (!G->dmem) return MANTRA_E_NOMEM;
+    G->b_dmem = total;
+    size_t off = 0;
+    for (int k = 0; k < SA_COUNT; ++k) {
+        char* p = (char*)G->dmem + off;
+        if (H.len[k]) CU(cudaMemcpyAsync(p, H.arr[k], H.len[k] * 4, cudaMemcpyHostToDevice, st));
+        *dst[k] = (const uint32_t*)p;
+        off += al256((H.len[k] + 1) * 4);
+    }
+    DirTimes dt{};
+    for (uint32_t j = 1; j < nb; ++j) dt.t[j] = H.arr[SA_ST_T][(size_t)j * H.m / nb];   // m > n here
+    char* base = (char*)G->dmem;
+    G->dg.n = H.n; G->dg.m = H.m; G->dg.A = H.A;
+    G->dg.out_vn = (const uint2*)(base + o_vn);
+    G->dg.in_out = (const uint32_t*)(base + o_io);
+    G->dg.out_pend = (const uint32_t*)(base + o_pe);
+    G->dg.dir = (const uint2*)(base + o_dir);
+    G->dg.dir_t = (const uint32_t*)(base + o_dt);
+    G->dg.dir_n = nb;
+    CU(launch_edge_maps(G->dg, dt, (uint2*)(base + o_vn), (uint32_t*)(base + o_io), (uint32_t*)(base + o_pe),
+                        (uint2*)(base + o_dir), (uint32_t*)(base + o_dt), st));
+    CU(cudaStreamSynchronize(st));
+    G->dg.out_loff = reinterpret_cast<const unsigned short*>(loff_words);
+    G->n = H.n; G->m = H.m; G->A = H.A; G->n_uedge = H.n_uedge;
+    G->self_loops = H.self_loops; G->duplicates = H.duplicates;
+    G->dg.n = H.n; G->dg.A = H.A; G->dg.m = H.m; G->dg.n_uedge = H.n_uedge;
+    G->dg.cbound = H.cbound; G->dg.max_slot_in = H.max_slot_in; G->dg.max_vslots = H.max_vslots;
+    return MANTRA_OK;
+}
+
+
+// The stream's waves for k_sweep, where its shared-memory state can hold the
+// graph: every vertex 4 bytes.  Streams with more than 16,384 edges in one time
+// step have none, nor have those whose waves would hold fewer than two edges
+// (a hub on every edge), where the sweep has no parallelism.  Nor have streams
+// under 2^16 edges: k_pfm_cta takes 0.1 us a sample there, and the cut would be
+// a tenth of the load.  MANTRA_PFM_KERNEL=sweep at the load lifts the last two.
+int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
+    const uint32_t m = G->m;
+    const char* env = std::getenv("MANTRA_PFM_KERNEL");
+    const bool force = env && std::strcmp(env, "sweep") == 0;
+    if (m < (force ? 1u : 1u << 16) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
+    const size_t bytes = wave_tmp_bytes(m, G->A);
+    char* tmp = (char*)pool.get(bytes);
+    if (!tmp) return MANTRA_E_NOMEM;
+    uint32_t head[2] = {0, 1};
+    int rc = MANTRA_OK;
+    if (launch_wave_cut(G->dg, tmp, st) != cudaSuccess ||
+        cudaMemcpyAsync(head, tmp, sizeof head, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        rc = MANTRA_E_CUDA;
+    if (rc == MANTRA_OK && head[1] == 0 && (force || (uint64_t)head[0] * 2 <= (uint64_t)m)) {
+        G->b_wmem = wave_bytes(head[0]);
+        G->wmem = pool.get(G->b_wmem);
+        if (!G->wmem) {
+            rc = MANTRA_E_NOMEM;
+        } else if (launch_wave_fill(&G->dg, tmp, head[0], (char*)G->wmem, st) != cudaSuccess ||
+                   cudaStreamSynchronize(st) != cudaSuccess) {
+            rc = MANTRA_E_CUDA;
+        }
+    }
+    pool.put(tmp, bytes);
+    return rc;
+}
 
 // Per-problem result slot of a tick: search counters, device status word,
 // and the round reduction's outputs.
@@ -249,6 +286,13 @@ struct Engine {
     std::map<uint64_t, int> hop_occ;       // (shape, shared nodes) -> CTAs per SM
     int tick_hop_nt = 256, tick_hop_sm = 0, tick_hop_cls = 0;
     uint32_t tick_hop_n = 0;
+    // pfm sweeps (k_sweep): a region per resident CTA (one warp, 32 samples);
+    // shared memory sized by the tick's graphs
+    char* sw_mem = nullptr; SweepWs sws{}; uint32_t sw_n = 0, sw_m = 0;
+    int sw_regions = 0, tick_sw_cls = 0;
+    uint32_t tick_sw_n = 0;
+    std::map<uint32_t, int> sw_occ;        // shared nodes -> CTAs per SM
+    bool tick_s = false;
     bool tick_b = false, tick_h = false, tick_p = false;   // kernel families with samples in the current tick
     char* pfm_mem = nullptr; PfmWs pws{}; int pfm_grid = 0; uint32_t pfm_n = 0, pfm_lcap = 0; uint64_t pfm_warps = 0;
     // pfm, one CTA per sample: shapes 0 = 256, 1 = 512 threads; modes 0 = state
@@ -263,7 +307,7 @@ struct Engine {
     uint32_t cap = 0;
     char* tab_h = nullptr; char* tab_d = nullptr; size_t tab_bytes = 0;
     char* slot_h = nullptr; char* slot_d = nullptr;
-    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_uh = 0, o_th = 0, o_ri = 0, o_rs = 0;
+    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_uh = 0, o_th = 0, o_us = 0, o_ts = 0, o_ri = 0, o_rs = 0;
     int red_grid = 0;
     // captured ticks, by launch configuration (tick_key)
     std::map<int, cudaGraphExec_t> gexec;
@@ -306,11 +350,26 @@ struct Engine {
         if (tick_b) key |= (shape_of(tick_bfs_nt) << 3) | (tick_bfs_sm << 5);
         if (tick_h) key |= (shape_of(tick_hop_nt) << 6) | (tick_hop_sm << 8) | ((tick_hop_sm ? tick_hop_cls : 0) << 13);
         if (tick_p) key |= ((tick_cta ? 1 : 0) << 9) | ((tick_pc_nt == 256 ? 0 : 1) << 10) | (tick_pc_sm << 11);
+        if (tick_s) key |= (1 << 21) | (tick_sw_cls << 22);
         return key;
     }
 
-    // Table block layout: header | work counters | unit starts (bfs, pfm, hop) |
-    // tasks (bfs, pfm, hop) | reduction items | reduction row starts.
+    // A node count rounded up by at most an eighth, and the number of its step:
+    // shared-memory state is sized in these steps, so that a tick's launch
+    // configurations (captured graphs) stay few.
+    static uint32_t node_step(uint32_t n, int* cls) {
+        uint32_t nq = 64;
+        int c = 0;
+        for (uint32_t step = 8; nq < n && c < 255; ++c) {
+            nq += step;
+            if (nq >= 16 * step) step *= 2;
+        }
+        *cls = c;
+        return nq;
+    }
+
+    // Table block layout: header | work counters | unit starts and tasks (bfs, pfm,
+    // hop, sweep) | reduction items | reduction row starts.
     int ensure_tables(uint32_t need) {
         if (tab_h && need <= cap) return MANTRA_OK;
         uint32_t nc = std::max<uint32_t>(64, cap);
@@ -320,14 +379,16 @@ struct Engine {
         if (slot_h) { cudaFreeHost(slot_h); slot_h = nullptr; }
         if (slot_d) { cudaFree(slot_d); slot_d = nullptr; }
         size_t o = 0;
-        o_hdr = o;  o = al256(o + 16);
-        o_work = o; o = al256(o + 24);
+        o_hdr = o;  o = al256(o + 20);
+        o_work = o; o = al256(o + 32);
         o_ub = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_up = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_tb = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_tp = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_uh = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_th = o;   o = al256(o + (size_t)nc * sizeof(Task));
+        o_us = o;   o = al256(o + (size_t)(nc + 1) * 8);
+        o_ts = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_ri = o;   o = al256(o + (size_t)nc * sizeof(ReduceItem));
         o_rs = o;   o = al256(o + (size_t)(nc + 1) * 4);
         tab_bytes = o;
@@ -530,12 +591,49 @@ struct Engine {
         return MANTRA_OK;
     }
 
+    // pfm sweeps: one region per resident CTA of a small graph, at most 16 GB or a
+    // tenth of free memory.
+    int ensure_sweep(uint32_t n, uint32_t m) {
+        if (sw_mem && n <= sw_n && m <= sw_m) return MANTRA_OK;
+        n = std::max(n, sw_n);
+        m = std::max(m, sw_m);
+        if (sw_mem) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_mem); sw_mem = nullptr; }
+        CU(sweep_configure(smem_optin - sweep_static_smem()));
+        const size_t region = sweep_region_bytes(n, m, &sws);
+        const size_t budget = std::min<size_t>((size_t)16 << 30, free_device_bytes() / 10);
+        const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 32, budget / region));
+        if (cudaMalloc(&sw_mem, (size_t)grid * region) != cudaSuccess) { sw_mem = nullptr; return MANTRA_E_NOMEM; }
+        sws.base = sw_mem;
+        sws.stride = region;
+        sw_regions = grid;
+        sw_n = n; sw_m = m;
+        invalidate_graph();
+        return MANTRA_OK;
+    }
+
+    // CTAs of k_sweep per SM with nsm nodes in shared memory; 0: they do not fit.
+    int sweep_per_sm(uint32_t nsm) {
+        const size_t smem = sweep_smem_bytes(nsm);
+        if (smem + sweep_static_smem() > smem_optin) return 0;
+        auto it = sw_occ.find(nsm);
+        if (it == sw_occ.end()) {
+            int per = 0;
+            if (sweep_configure(smem_optin - sweep_static_smem()) != cudaSuccess ||
+                sweep_blocks_per_sm(smem, &per) != cudaSuccess)
+                per = 0;
+            it = sw_occ.emplace(nsm, per).first;
+        }
+        return it->second;
+    }
+
+    int sweep_grid(uint32_t nsm) { return std::min(sw_regions, sweep_per_sm(nsm) * num_sms); }
+
     // The tick as stream work: tables up, slots cleared, both search
     // families on two streams, the round reduction, slots down.
     int enqueue(bool wide) {
         CU(cudaMemcpyAsync(tab_d, tab_h, tab_bytes, cudaMemcpyHostToDevice, sa));
         CU(cudaMemsetAsync(slot_d, 0, (size_t)cap * SLOT_BYTES, sa));
-        if (tick_p) {
+        if (tick_p || tick_s) {
             CU(cudaEventRecord(ev_fork, sa));
             CU(cudaStreamWaitEvent(sb, ev_fork, 0));
         }
@@ -557,22 +655,26 @@ struct Engine {
                           bfs_grids[shape_of(tick_bfs_nt)][tick_bfs_sm], tick_bfs_sm ? bfs_smem : 0, wide, sa));
         }
         if (tick_b || tick_h) CU(cudaEventRecord(e_b1, sa));
+        if (tick_p || tick_s) CU(cudaEventRecord(e_p0, sb));
+        if (tick_s) {
+            SweepWs w = sws;
+            w.n_smem = tick_sw_n;
+            CU(launch_sweep((const Task*)(tab_d + o_ts), (const uint64_t*)(tab_d + o_us), hdr + 4, work + 3, w,
+                            sweep_grid(tick_sw_n), sb));
+        }
         if (tick_p && tick_cta) {
-            CU(cudaEventRecord(e_p0, sb));
             PfmCtaWs w = pcws;
             w.nt = tick_pc_nt;
             w.fa_in_smem = tick_pc_sm == 1 ? 1 : (tick_pc_sm == 3 ? 2 : 0);
             w.stage_cap = tick_pc_sm == 2 ? PFM_STAGE_CAP : 0u;
             CU(launch_pfm_cta((const Task*)(tab_d + o_tp), (const uint64_t*)(tab_d + o_up), hdr + 1, work + 1, w,
                               pc_grids[tick_pc_nt == 256 ? 0 : 1][tick_pc_sm], sb));
-            CU(cudaEventRecord(e_p1, sb));
         } else if (tick_p) {
-            CU(cudaEventRecord(e_p0, sb));
             CU(launch_pfm((const Task*)(tab_d + o_tp), (const uint64_t*)(tab_d + o_up), hdr + 1, work + 1, pws,
                           pfm_grid, wide, sb));
-            CU(cudaEventRecord(e_p1, sb));
         }
-        if (tick_p) {
+        if (tick_p || tick_s) {
+            CU(cudaEventRecord(e_p1, sb));
             CU(cudaEventRecord(ev_join, sb));
             CU(cudaStreamWaitEvent(sa, ev_join, 0));
         }
@@ -679,6 +781,42 @@ bool pfm_use_cta() {
     return !(env && std::strcmp(env, "lane") == 0);
 }
 
+// Whether the sweep (k_sweep) can take an item's samples.
+bool can_sweep(const TickItem& it) {
+    const Job& j = it.job;
+    return j.opt == MANTRA_PFM && !j.ob && !j.rtb && !j.stats && it.G->dg.n_waves > 0;
+}
+
+// Whether a tick's pfm samples take the sweep where they can.  The sweep's time
+// is that of the longest stream (one warp, 75 ns a wave), or its warps' waves
+// spread over the resident CTAs (both a third longer when the GPU is full); the
+// CTA kernel's, a graph-sized latency and a share per sample.  Measured (ms,
+// sweep / CTA): n = 20,000 bursty 231 samples 2.97 / 0.79, 42,000 samples 14.9 /
+// 33.4; n = 5,000 231: 1.16 / 0.22, 10,000: 1.40 / 2.53; n = 1,000 2,000: 0.60 /
+// 0.37; n = 50,000 uniform 231: 6.8 / 2.0, 8,000: 17.9 / 41.0.
+// MANTRA_PFM_KERNEL=sweep|cta|lane forces one of them.
+bool use_sweep(Engine& E, const std::vector<TickItem>& items) {
+    uint32_t n = 0;
+    double longest = 0, waves = 0, base = 0, samples = 0;
+    for (const TickItem& it : items) {
+        if (!can_sweep(it)) continue;
+        const double w = 75e-6 * it.G->dg.n_waves, m = it.G->m, r = (double)it.job.count;
+        n = std::max(n, it.G->n);
+        longest = std::max(longest, w);
+        waves += w * std::ceil(r / 32.0);
+        base = std::max(base, 0.08 + 1.2e-6 * m);
+        samples += r * (8e-5 + 1.4e-9 * m);
+    }
+    if (!n) return false;
+    if (const char* env = std::getenv("MANTRA_PFM_KERNEL")) {
+        if (std::strcmp(env, "lane") == 0 || std::strcmp(env, "cta") == 0) return false;
+        if (std::strcmp(env, "sweep") == 0) return true;
+    }
+    int cls = 0;
+    const int per = std::max(1, E.sweep_per_sm(Engine::node_step(n, &cls)));
+    return 0.2 + 1.35 * std::max(longest, waves / ((double)per * E.num_sms)) < base + samples;
+}
+
 // One tick over `items` (narrow kernels, captured graph), or with `wide` the
 // 128-bit kernels launched directly.  Fills each item's ctr/status pointers.
 int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
@@ -692,8 +830,16 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     uint32_t hn = 0, hA = 0;
     uint64_t hsamples = 0;
     const mantra_graph* gh = nullptr;   // the tick's largest k_hop graph
-    for (const TickItem& it : items) {
-        if (it.job.opt == MANTRA_PFM) {
+    bool any_s = false;
+    uint32_t sn = 0, smx = 0;
+    std::vector<char> sweep(k, 0);
+    const bool sweeps = !wide && use_sweep(E, items);
+    for (uint32_t x = 0; x < k; ++x) {
+        const TickItem& it = items[x];
+        if (sweeps && can_sweep(it)) {
+            sweep[x] = 1;
+            any_s = true; sn = std::max(sn, it.G->n); smx = std::max(smx, it.G->m);
+        } else if (it.job.opt == MANTRA_PFM) {
             any_p = true; pn = std::max(pn, it.G->n); plc = std::max(plc, it.G->dg.cbound);
             pz = std::max(pz, it.G->dg.max_vslots);
             if (!gp || it.G->n > gp->n) gp = it.G;
@@ -709,9 +855,19 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             dl |= it.job.ob || it.job.rtb;
         }
     }
-    E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p;
+    E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p; E.tick_s = any_s;
     const bool cta = any_p && !wide && pfm_use_cta();
     if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
+    if (any_s) {
+        if ((rc = E.ensure_sweep(sn, smx)) != MANTRA_OK) return rc;
+        E.tick_sw_n = Engine::node_step(sn, &E.tick_sw_cls);
+        // near the limit the step may not fit: the graphs' own size then (a graph with
+        // waves fits), captured as the last step
+        if (!E.sweep_grid(E.tick_sw_n)) {
+            E.tick_sw_n = E.sw_n;
+            E.tick_sw_cls = 255;
+        }
+    }
     if (any_b && (rc = E.ensure_bfs(bn, bA, bz, dl)) != MANTRA_OK) return rc;
     if (any_p && cta && (rc = E.ensure_pfm_cta(pn, plc)) != MANTRA_OK) return rc;
     if (any_p && !cta && (rc = E.ensure_pfm(pn, plc, pwarps)) != MANTRA_OK) return rc;
@@ -730,12 +886,8 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     // mantra_tune's choice for the graph comes first; MANTRA_BFS_NT=256|512|1024 and
     // MANTRA_BFS_SMEM=0|1 force them.
     if (any_h) {
-        uint32_t nq = 64;                        // shared nodes: the tick's largest graph, rounded up by at most 1/8
         int cls = 0;
-        for (uint32_t step = 8; nq < hn && cls < 255; ++cls) {
-            nq += step;
-            if (nq >= 16 * step) step *= 2;
-        }
+        const uint32_t nq = Engine::node_step(hn, &cls);
         auto grid = [&](int nt, int sm) { return E.hop_grid(nt, sm ? nq : 0, E.hop_regions); };
         int nt = 1024, sm = 0;
         if (hsamples <= 2ull * (uint64_t)E.num_sms) {
@@ -802,21 +954,27 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     u64* work = (u64*)(E.tab_h + E.o_work);
     uint64_t* ub = (uint64_t*)(E.tab_h + E.o_ub);
     uint64_t* up = (uint64_t*)(E.tab_h + E.o_up);
+    uint64_t* us = (uint64_t*)(E.tab_h + E.o_us);
+    Task* tsw = (Task*)(E.tab_h + E.o_ts);
     uint64_t* uh = (uint64_t*)(E.tab_h + E.o_uh);
     Task* th = (Task*)(E.tab_h + E.o_th);
     Task* tb = (Task*)(E.tab_h + E.o_tb);
     Task* tp = (Task*)(E.tab_h + E.o_tp);
     ReduceItem* ri = (ReduceItem*)(E.tab_h + E.o_ri);
     uint32_t* rs = (uint32_t*)(E.tab_h + E.o_rs);
-    uint32_t nb = 0, np = 0, nr = 0, nh = 0;
-    ub[0] = 0; up[0] = 0; uh[0] = 0; rs[0] = 0;
+    uint32_t nb = 0, np = 0, nr = 0, nh = 0, ns = 0;
+    ub[0] = 0; up[0] = 0; uh[0] = 0; us[0] = 0; rs[0] = 0;
     for (uint32_t x = 0; x < k; ++x) {
         TickItem& it = items[x];
         char* slot = E.slot_d + (size_t)x * SLOT_BYTES;
         it.job.ctr = (u64*)slot;
         it.job.status = (int*)(slot + SLOT_STATUS);
         Task t{it.G->dg, it.job};
-        if (it.job.opt == MANTRA_PFM) {
+        if (sweep[x]) {
+            tsw[ns] = t;
+            us[ns + 1] = us[ns] + (it.job.count + 31) / 32;
+            ++ns;
+        } else if (it.job.opt == MANTRA_PFM) {
             tp[np] = t;
             up[np + 1] = up[np] + (cta ? it.job.count : (it.job.count + 31) / 32);
             ++np;
@@ -832,14 +990,14 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             ++nr;
         }
     }
-    hdr[0] = nb; hdr[1] = np; hdr[2] = nr; hdr[3] = nh;
-    work[0] = 0; work[1] = 0; work[2] = 0;
+    hdr[0] = nb; hdr[1] = np; hdr[2] = nr; hdr[3] = nh; hdr[4] = ns;
+    work[0] = 0; work[1] = 0; work[2] = 0; work[3] = 0;
     if ((rc = E.launch_tick(wide)) != MANTRA_OK) return rc;
     CU(cudaStreamSynchronize(E.sa));
     out->slot.resize(k);
     for (uint32_t x = 0; x < k; ++x) out->slot[x] = E.slot_h + (size_t)x * SLOT_BYTES;
     out->had_bfs = nb + nh > 0;
-    out->had_pfm = np > 0;
+    out->had_pfm = np + ns > 0;
     if (E.last_tick_graph) {
         // a graph tick is timed as a whole: table upload, searches, reduction, readback
         const double t = elapsed_ms(E.e_t0, E.e_t1);
@@ -851,7 +1009,9 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     }
     for (uint32_t x = 0; x < k; ++x) {
         const u64* c = (const u64*)out->slot[x];
-        if (items[x].job.opt == MANTRA_PFM)
+        if (sweep[x])
+            log_item(items[x], "k_sweep", wide, 32, 0, c, out->pfm_ms);
+        else if (items[x].job.opt == MANTRA_PFM)
             log_item(items[x], cta ? "k_pfm_cta" : "k_pfm", wide, cta ? E.tick_pc_nt : 32, cta ? E.tick_pc_sm : 0, c,
                      out->pfm_ms);
         else if (!wide && on_hop(items[x].G, items[x].job))
@@ -1465,7 +1625,8 @@ int mantra_graph_load(const uint32_t* u, const uint32_t* v, const uint32_t* t, u
         std::lock_guard<std::mutex> lock(E->mu);
         StoreHost H;
         rc = E->store.build(u, v, t, m, n, &H);
-        if (rc == MANTRA_OK) rc = upload_store(H, G, E->sa);
+        if (rc == MANTRA_OK) rc = upload_store(H, G, E->pool, E->sa);
+        if (rc == MANTRA_OK) rc = build_waves(G, E->smem_optin, E->pool, E->sa);
         E->store.trim();
     }
     if (rc != MANTRA_OK) { mantra_graph_free(G); return rc; }
@@ -1510,9 +1671,11 @@ void mantra_graph_free(mantra_graph* g) {
         std::lock_guard<std::mutex> lock(E->mu);
         cudaStreamSynchronize(E->sa);
         cudaStreamSynchronize(E->sb);
-        cudaFree(g->dmem);
-    } else if (g->dmem) {
-        cudaFree(g->dmem);
+        E->pool.put(g->dmem, g->b_dmem);
+        E->pool.put(g->wmem, g->b_wmem);
+    } else {
+        if (g->dmem) cudaFree(g->dmem);
+        if (g->wmem) cudaFree(g->wmem);
     }
     delete g;
 }

@@ -1272,21 +1272,22 @@ __global__ void k_edge_maps(DevGraph g, uint2* out_vn, uint32_t* in_out, uint32_
 }
 
 // dir[b n + v]: the edges of v's out-row that bucket b of the times spans.
-__global__ void k_edge_dir(DevGraph g, uint2* dir) {
+__global__ void k_edge_dir(DevGraph g, DirTimes dt, uint2* dir, uint32_t* dir_t) {
     const uint64_t x = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (x < 32) dir_t[x] = dt.t[x];
     if (x >= (uint64_t)g.n * g.dir_n) return;
     const uint32_t b = (uint32_t)(x / g.n), v = (uint32_t)(x - (uint64_t)b * g.n);
     const uint32_t r0 = g.out_ptr[v], r1 = g.out_ptr[v + 1];
-    const uint32_t lo = lower_bound_u32(g.out_t, r0, r1, g.dir_t[b]);
-    dir[x] = make_uint2(lo, b + 1 < g.dir_n ? lower_bound_u32(g.out_t, lo, r1, g.dir_t[b + 1]) : r1);
+    const uint32_t lo = lower_bound_u32(g.out_t, r0, r1, dt.t[b]);
+    dir[x] = make_uint2(lo, b + 1 < g.dir_n ? lower_bound_u32(g.out_t, lo, r1, dt.t[b + 1]) : r1);
 }
 
-// Fills out_vn, in_out, out_pend and dir of g (whose other arrays are in place).
-cudaError_t launch_edge_maps(const DevGraph& g, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend, uint2* dir,
-                             cudaStream_t st) {
+// Fills out_vn, in_out, out_pend, dir and dir_t of g (whose other arrays are in place).
+cudaError_t launch_edge_maps(const DevGraph& g, const DirTimes& dt, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend,
+                             uint2* dir, uint32_t* dir_t, cudaStream_t st) {
     if (g.m) k_edge_maps<<<(g.m + 255) / 256, 256, 0, st>>>(g, out_vn, in_out, out_pend);
     const uint64_t d = (uint64_t)g.n * g.dir_n;
-    k_edge_dir<<<(unsigned)((d + 255) / 256), 256, 0, st>>>(g, dir);
+    k_edge_dir<<<(unsigned)((d + 255) / 256), 256, 0, st>>>(g, dt, dir, dir_t);
     return cudaGetLastError();
 }
 

@@ -73,6 +73,27 @@ struct DevGraph {
                                  // dir_t[b + 1] (the last bucket: to the row's end)
     const uint32_t* dir_t;       // dir_n bucket times, ascending, the first 0
     uint32_t dir_n;              // buckets of the times (at most 32)
+    // the stream cut into waves of at most 32 independent edges (k_sweep.cu; none: n_waves = 0)
+    uint32_t n_waves;            // a multiple of WAVE_BATCH
+    const uint2* wave_uv;        // 32 per wave: u, v (padding: n, n)
+    const uint2* wave_at;        // 32 per wave: the head's slot, t
+    const uint2* wave_info;      // per batch: its last time; not 0: a wave of it has flags
+    const uint32_t* wave_t;      // per wave: its last time
+    const uint32_t* wave_fl;     // per wave: WAVE_BIG, WAVE_LAST, WAVE_SEVERAL
+};
+
+// Stream edges per part of the wave cut (a thread each: 512 made a load of 125,000
+// edges 0.25 ms longer, 128 a sweep 2 % longer); waves of one time step at most; waves
+// per batch.  Flags of a wave: part of a time step of several waves, the last of
+// them; an edge's head slot has several in-edges.
+constexpr uint32_t WAVE_CUT = 128, WAVE_STEP = 512, WAVE_BATCH = 8;
+constexpr uint32_t WAVE_BIG = 1u, WAVE_LAST = 2u, WAVE_SEVERAL = 4u;
+
+// The waves' arrays while they are filled (see DevGraph).
+struct WaveArrays {
+    uint32_t n_waves;
+    uint2 *uv, *at, *info;
+    uint32_t *t, *fl;
 };
 
 // Largest number of arrival slots of one vertex for the CTA pfm kernel's
@@ -779,6 +800,16 @@ struct HopWs {
     uint32_t n_smem;     // nodes whose next-level arrivals are in dynamic shared memory (0: in the region)
 };
 
+// Per-warp scratch of the pfm sweep over the stream (one region per CTA).
+struct SweepWs {
+    char* base;          // CTA b uses base + b * stride
+    size_t stride;
+    size_t o_log, o_arr, o_stp, o_path, o_pathe, o_cv, o_co, o_ck, o_sig;
+    uint32_t n_smem;     // nodes of the shared-memory state
+    uint32_t path_cap;   // vertices of a path; longer: the sample goes to the overflow list
+    uint32_t cone_cap;   // vertices that lead to z of a sample with a choice; more: the overflow list
+};
+
 // Per-warp scratch of the pfm search kernel.
 struct PfmWs {
     char* base;          // warp w uses base + w * stride
@@ -820,9 +851,24 @@ cudaError_t hop_configure(size_t smem);
 cudaError_t hop_blocks_per_sm(int nt, bool first_in_smem, size_t smem, int* out);
 cudaError_t launch_hop(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
                        const HopWs& ws, int grid, cudaStream_t st);
-// Fills out_vn, in_out, out_pend and dir of g (whose other arrays are in place).
-cudaError_t launch_edge_maps(const DevGraph& g, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend, uint2* dir,
-                             cudaStream_t st);
+// Fills out_vn, in_out, out_pend, dir and dir_t of g (whose other arrays are in place).
+struct DirTimes { uint32_t t[32]; };
+cudaError_t launch_edge_maps(const DevGraph& g, const DirTimes& dt, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend,
+                             uint2* dir, uint32_t* dir_t, cudaStream_t st);
+size_t sweep_region_bytes(uint32_t n, uint32_t m, SweepWs* ws);
+size_t sweep_smem_bytes(uint32_t n);
+size_t sweep_static_smem();
+cudaError_t sweep_configure(size_t smem);
+cudaError_t sweep_blocks_per_sm(size_t smem, int* out);
+cudaError_t launch_sweep(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
+                         const SweepWs& ws, int grid, cudaStream_t st);
+// The waves of a graph: the cut into tmp (wave_tmp_bytes), whose first
+// two words then hold their number and whether a time step has too many edges
+// (no waves); then the fill.
+size_t wave_tmp_bytes(uint32_t m, uint32_t A);
+cudaError_t launch_wave_cut(const DevGraph& g, char* tmp, cudaStream_t st);
+size_t wave_bytes(uint32_t total);
+cudaError_t launch_wave_fill(DevGraph* g, char* tmp, uint32_t total, char* mem, cudaStream_t st);
 size_t pfm_region_bytes(uint32_t n, uint32_t list_cap, PfmWs* ws);
 int pfm_threads();
 cudaError_t launch_pfm(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
