@@ -290,6 +290,7 @@ struct Engine {
     // shared memory sized by the tick's graphs
     char* sw_mem = nullptr; SweepWs sws{}; uint32_t sw_n = 0, sw_m = 0;
     int sw_regions = 0, tick_sw_cls = 0;
+    uint32_t* sw_order = nullptr; uint64_t sw_order_cap = 0; bool tick_sw_order = false;
     uint32_t tick_sw_n = 0;
     std::map<uint32_t, int> sw_occ;        // shared nodes -> CTAs per SM
     bool tick_s = false;
@@ -350,7 +351,7 @@ struct Engine {
         if (tick_b) key |= (shape_of(tick_bfs_nt) << 3) | (tick_bfs_sm << 5);
         if (tick_h) key |= (shape_of(tick_hop_nt) << 6) | (tick_hop_sm << 8) | ((tick_hop_sm ? tick_hop_cls : 0) << 13);
         if (tick_p) key |= ((tick_cta ? 1 : 0) << 9) | ((tick_pc_nt == 256 ? 0 : 1) << 10) | (tick_pc_sm << 11);
-        if (tick_s) key |= (1 << 21) | (tick_sw_cls << 22);
+        if (tick_s) key |= (1 << 21) | (tick_sw_cls << 22) | ((tick_sw_order ? 1 : 0) << 30);
         return key;
     }
 
@@ -611,6 +612,20 @@ struct Engine {
         return MANTRA_OK;
     }
 
+    // Places for the ordered samples of a tick's sweep units; none past 2^24 samples
+    // (64 MB), where the units are taken as they come.
+    int ensure_sweep_order(uint64_t units) {
+        tick_sw_order = units > 1 && units * 32 <= (1ull << 24);
+        if (!tick_sw_order || units * 32 <= sw_order_cap) return MANTRA_OK;
+        uint64_t cap = std::max<uint64_t>(sw_order_cap, 1u << 16);
+        while (cap < units * 32) cap *= 2;
+        if (sw_order) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_order); sw_order = nullptr; sw_order_cap = 0; }
+        if (cudaMalloc((void**)&sw_order, cap * 4) != cudaSuccess) { sw_order = nullptr; return MANTRA_E_NOMEM; }
+        sw_order_cap = cap;
+        invalidate_graph();
+        return MANTRA_OK;
+    }
+
     // CTAs of k_sweep per SM with nsm nodes in shared memory; 0: they do not fit.
     int sweep_per_sm(uint32_t nsm) {
         const size_t smem = sweep_smem_bytes(nsm);
@@ -659,6 +674,7 @@ struct Engine {
         if (tick_s) {
             SweepWs w = sws;
             w.n_smem = tick_sw_n;
+            w.order = tick_sw_order ? sw_order : nullptr;
             CU(launch_sweep((const Task*)(tab_d + o_ts), (const uint64_t*)(tab_d + o_us), hdr + 4, work + 3, w,
                             sweep_grid(tick_sw_n), sb));
         }
@@ -789,11 +805,11 @@ bool can_sweep(const TickItem& it) {
 
 // Whether a tick's pfm samples take the sweep where they can.  The sweep's time
 // is that of the longest stream (one warp, 75 ns a wave), or its warps' waves
-// spread over the resident CTAs (both a third longer when the GPU is full); the
-// CTA kernel's, a graph-sized latency and a share per sample.  Measured (ms,
-// sweep / CTA): n = 20,000 bursty 231 samples 2.97 / 0.79, 42,000 samples 14.9 /
-// 33.4; n = 5,000 231: 1.16 / 0.22, 10,000: 1.40 / 2.53; n = 1,000 2,000: 0.60 /
-// 0.37; n = 50,000 uniform 231: 6.8 / 2.0, 8,000: 17.9 / 41.0.
+// spread over the resident CTAs (ordered samples skip part of them, about what a
+// full GPU adds); the CTA kernel's, a graph-sized latency and a share per sample.
+// Measured (ms, sweep / CTA): n = 20,000 bursty 231 samples 2.7 / 0.79, 42,000
+// samples 9.1 / 33.4; n = 5,000 231: 1.1 / 0.22, 10,000: 1.39 / 2.53; n = 1,000
+// 2,000: 0.54 / 0.37; n = 50,000 uniform 231: 5.4 / 2.0, 8,000: 12.3 / 41.0.
 // MANTRA_PFM_KERNEL=sweep|cta|lane forces one of them.
 bool use_sweep(Engine& E, const std::vector<TickItem>& items) {
     uint32_t n = 0;
@@ -814,7 +830,7 @@ bool use_sweep(Engine& E, const std::vector<TickItem>& items) {
     }
     int cls = 0;
     const int per = std::max(1, E.sweep_per_sm(Engine::node_step(n, &cls)));
-    return 0.2 + 1.35 * std::max(longest, waves / ((double)per * E.num_sms)) < base + samples;
+    return 0.2 + std::max(1.3 * longest, waves / ((double)per * E.num_sms)) < base + samples;
 }
 
 // One tick over `items` (narrow kernels, captured graph), or with `wide` the
@@ -832,6 +848,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     const mantra_graph* gh = nullptr;   // the tick's largest k_hop graph
     bool any_s = false;
     uint32_t sn = 0, smx = 0;
+    uint64_t sunits = 0;
     std::vector<char> sweep(k, 0);
     const bool sweeps = !wide && use_sweep(E, items);
     for (uint32_t x = 0; x < k; ++x) {
@@ -839,6 +856,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         if (sweeps && can_sweep(it)) {
             sweep[x] = 1;
             any_s = true; sn = std::max(sn, it.G->n); smx = std::max(smx, it.G->m);
+            sunits += (it.job.count + 31) / 32;
         } else if (it.job.opt == MANTRA_PFM) {
             any_p = true; pn = std::max(pn, it.G->n); plc = std::max(plc, it.G->dg.cbound);
             pz = std::max(pz, it.G->dg.max_vslots);
@@ -860,6 +878,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
     if (any_s) {
         if ((rc = E.ensure_sweep(sn, smx)) != MANTRA_OK) return rc;
+        if ((rc = E.ensure_sweep_order(sunits)) != MANTRA_OK) return rc;
         E.tick_sw_n = Engine::node_step(sn, &E.tick_sw_cls);
         // near the limit the step may not fit: the graphs' own size then (a graph with
         // waves fits), captured as the last step

@@ -805,6 +805,7 @@ struct SweepWs {
     char* base;          // CTA b uses base + b * stride
     size_t stride;
     size_t o_log, o_arr, o_stp, o_path, o_pathe, o_cv, o_co, o_ck, o_sig;
+    uint32_t* order;     // or nullptr: the units' samples (32 places per unit), see k_sweep_order
     uint32_t n_smem;     // nodes of the shared-memory state
     uint32_t path_cap;   // vertices of a path; longer: the sample goes to the overflow list
     uint32_t cone_cap;   // vertices that lead to z of a sample with a choice; more: the overflow list
