@@ -137,11 +137,12 @@ typedef struct {
                                 edges_scanned / 32 (the edge record, shared by 32 samples) + 24 *
                                 sigma_adds (sigma(u) read, sigma(v) read-modify-write) */
     uint64_t frontier_vertices; /* F (above) */
-    uint64_t edges_expanded; /* pfm, one CTA per sample (the default pfm kernel): out-edges walked by
-                                the earliest-arrival rounds plus prefix-foremost DAG edges walked by the
-                                path-count pass; that kernel's own algorithmic bytes are 12 per walked
-                                edge (8 B record, 4 B arrival test or count read) + 24 * sigma_adds.
-                                0 for sh / sfm and for the stream-scan kernel */
+    uint64_t edges_expanded; /* pfm samples of the label-correcting search (k_pfm_cta): out-edges walked
+                                by the earliest-arrival rounds plus prefix-foremost DAG edges walked by
+                                the path-count pass, where there is one; that kernel's own algorithmic
+                                bytes are 12 per walked edge (8 B record, 4 B arrival test or count
+                                read) + 24 * sigma_adds.  0 for sh / sfm and for the kernels that pass
+                                over the time-sorted edges (k_sweep, k_scan, k_pfm) */
 } mantra_info;
 
 /* Output of mantra_temporal_stats (paper App. D, Algorithm 2). */

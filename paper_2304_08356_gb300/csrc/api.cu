@@ -34,6 +34,7 @@ struct Knobs {
     int pfm_nt = 0;      // pfm CTA size: 256 or 512
     int pfm_mode = -1;   // pfm arrival state: 1 shared memory, 0 global, 2 global with the out-edge tiles
                          // staged in shared memory by bulk copies
+    bool pfm_search = false;   // a probe of the two: pfm by the search (k_pfm_cta) whatever the rules say
 };
 
 // Out-edges per chunk the staged pfm variant copies into shared memory (the
@@ -47,7 +48,8 @@ struct mantra_graph {
     DevGraph dg{};
     void* dmem = nullptr;
     void* wmem = nullptr;   // waves of the stream (k_sweep), or none
-    size_t b_dmem = 0, b_wmem = 0;
+    void* smem = nullptr;   // k_scan's chunks of the stream, or none
+    size_t b_dmem = 0, b_wmem = 0, b_smem = 0;
     int device = 0;
     Knobs knobs;         // set by mantra_tune
 };
@@ -179,17 +181,23 @@ int upload_store(const StoreHost& H, mantra_graph* G, DevPool& pool, cudaStream_
 }
 
 
+// Whether nearly every arrival slot has one in-edge, so that hardly any way back
+// has a choice: one warp counts and draws the paths of such a sample in k_sweep and
+// k_scan, the whole CTA in k_pfm_cta.
+bool few_choices(const mantra_graph* G) { return (uint64_t)G->A * 100 >= (uint64_t)G->m * 97; }
+
 // The stream's waves for k_sweep, where its shared-memory state can hold the
 // graph: every vertex 4 bytes.  Streams with more than 16,384 edges in one time
 // step have none, nor have those whose waves would hold fewer than two edges
 // (a hub on every edge), where the sweep has no parallelism.  Nor have streams
 // under 2^16 edges: k_pfm_cta takes 0.1 us a sample there, and the cut would be
-// a tenth of the load.  MANTRA_PFM_KERNEL=sweep at the load lifts the last two.
+// a tenth of the load.  Nor graphs in which ways back have
+// choices (few_choices).  MANTRA_PFM_KERNEL=sweep at the load lifts the last three.
 int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
     const bool force = env && std::strcmp(env, "sweep") == 0;
-    if (m < (force ? 1u : 1u << 16) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
+    if (m < (force ? 1u : 1u << 16) || !(force || few_choices(G)) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
     const size_t bytes = wave_tmp_bytes(m, G->A);
     char* tmp = (char*)pool.get(bytes);
     if (!tmp) return MANTRA_E_NOMEM;
@@ -211,6 +219,34 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
     }
     pool.put(tmp, bytes);
     return rc;
+}
+
+// The stream's chunks for k_scan, where its shared-memory bits can hold the
+// graph, no time step exceeds a chunk, and few edges share an arrival slot
+// (MANTRA_PFM_KERNEL=scan at the load lifts the last).
+int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
+    const uint32_t m = G->m;
+    const char* env = std::getenv("MANTRA_PFM_KERNEL");
+    const bool force = env && std::strcmp(env, "scan") == 0;
+    if (m == 0 || !(force || few_choices(G)) || scan_smem_bytes(1024, G->n) > smem_optin) return MANTRA_OK;
+    const size_t nc = ((size_t)m + SCAN_CHUNK - 1) / SCAN_CHUNK;
+    G->b_smem = al256((size_t)m * 4) + al256((nc + 1) * 4) + 256;
+    G->smem = pool.get(G->b_smem);
+    if (!G->smem) return MANTRA_E_NOMEM;
+    uint32_t* slot = (uint32_t*)G->smem;
+    uint32_t* ptr = (uint32_t*)((char*)G->smem + al256((size_t)m * 4));
+    uint32_t* big = (uint32_t*)((char*)ptr + al256((nc + 1) * 4));
+    uint32_t flag = 1;
+    if (launch_scan_maps(G->dg, slot, ptr, big, st) != cudaSuccess ||
+        cudaMemcpyAsync(&flag, big, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return MANTRA_E_CUDA;
+    if (flag == 0) {
+        G->dg.st_slot = slot;
+        G->dg.scan_ptr = ptr;
+        G->dg.n_scan = (uint32_t)nc;
+    }
+    return MANTRA_OK;
 }
 
 // Per-problem result slot of a tick: search counters, device status word,
@@ -294,6 +330,12 @@ struct Engine {
     uint32_t tick_sw_n = 0;
     std::map<uint32_t, int> sw_occ;        // shared nodes -> CTAs per SM
     bool tick_s = false;
+    // pfm scans (k_scan): a region per resident CTA
+    char* sc_mem = nullptr; ScanWs scws{}; uint32_t sc_n = 0;
+    int sc_regions = 0, tick_sc_nt = 512, tick_sc_cls = 0;
+    uint32_t tick_sc_n = 0;
+    std::map<uint64_t, int> sc_occ;        // (threads, shared nodes) -> CTAs per SM
+    bool tick_n = false;
     bool tick_b = false, tick_h = false, tick_p = false;   // kernel families with samples in the current tick
     char* pfm_mem = nullptr; PfmWs pws{}; int pfm_grid = 0; uint32_t pfm_n = 0, pfm_lcap = 0; uint64_t pfm_warps = 0;
     // pfm, one CTA per sample: shapes 0 = 256, 1 = 512 threads; modes 0 = state
@@ -308,10 +350,10 @@ struct Engine {
     uint32_t cap = 0;
     char* tab_h = nullptr; char* tab_d = nullptr; size_t tab_bytes = 0;
     char* slot_h = nullptr; char* slot_d = nullptr;
-    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_uh = 0, o_th = 0, o_us = 0, o_ts = 0, o_ri = 0, o_rs = 0;
+    size_t o_hdr = 0, o_work = 0, o_ub = 0, o_up = 0, o_tb = 0, o_tp = 0, o_uh = 0, o_th = 0, o_us = 0, o_ts = 0, o_un = 0, o_tn = 0, o_ri = 0, o_rs = 0;
     int red_grid = 0;
     // captured ticks, by launch configuration (tick_key)
-    std::map<int, cudaGraphExec_t> gexec;
+    std::map<uint64_t, cudaGraphExec_t> gexec;
     bool use_graph = true;
     DevPool pool;
 
@@ -345,13 +387,14 @@ struct Engine {
 
     static int shape_of(int nt) { return nt == 256 ? 0 : (nt == 1024 ? 2 : 1); }
 
-    int tick_key() const {
+    uint64_t tick_key() const {
         // a family without samples is not launched; its launch choices are left out
-        int key = (tick_b ? 1 : 0) | (tick_h ? 2 : 0) | (tick_p ? 4 : 0);
+        uint64_t key = (tick_b ? 1 : 0) | (tick_h ? 2 : 0) | (tick_p ? 4 : 0);
         if (tick_b) key |= (shape_of(tick_bfs_nt) << 3) | (tick_bfs_sm << 5);
         if (tick_h) key |= (shape_of(tick_hop_nt) << 6) | (tick_hop_sm << 8) | ((tick_hop_sm ? tick_hop_cls : 0) << 13);
         if (tick_p) key |= ((tick_cta ? 1 : 0) << 9) | ((tick_pc_nt == 256 ? 0 : 1) << 10) | (tick_pc_sm << 11);
         if (tick_s) key |= (1 << 21) | (tick_sw_cls << 22) | ((tick_sw_order ? 1 : 0) << 30);
+        if (tick_n) key |= (1ull << 31) | ((uint64_t)tick_sc_cls << 32) | ((uint64_t)(tick_sc_nt == 1024) << 40);
         return key;
     }
 
@@ -370,7 +413,7 @@ struct Engine {
     }
 
     // Table block layout: header | work counters | unit starts and tasks (bfs, pfm,
-    // hop, sweep) | reduction items | reduction row starts.
+    // hop, sweep, scan) | reduction items | reduction row starts.
     int ensure_tables(uint32_t need) {
         if (tab_h && need <= cap) return MANTRA_OK;
         uint32_t nc = std::max<uint32_t>(64, cap);
@@ -380,14 +423,16 @@ struct Engine {
         if (slot_h) { cudaFreeHost(slot_h); slot_h = nullptr; }
         if (slot_d) { cudaFree(slot_d); slot_d = nullptr; }
         size_t o = 0;
-        o_hdr = o;  o = al256(o + 20);
-        o_work = o; o = al256(o + 32);
+        o_hdr = o;  o = al256(o + 24);
+        o_work = o; o = al256(o + 40);
         o_ub = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_up = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_tb = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_tp = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_uh = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_th = o;   o = al256(o + (size_t)nc * sizeof(Task));
+        o_un = o;   o = al256(o + (size_t)(nc + 1) * 8);
+        o_tn = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_us = o;   o = al256(o + (size_t)(nc + 1) * 8);
         o_ts = o;   o = al256(o + (size_t)nc * sizeof(Task));
         o_ri = o;   o = al256(o + (size_t)nc * sizeof(ReduceItem));
@@ -643,12 +688,44 @@ struct Engine {
 
     int sweep_grid(uint32_t nsm) { return std::min(sw_regions, sweep_per_sm(nsm) * num_sms); }
 
+    // pfm scans: one region per CTA of the largest grid (two per SM).
+    int ensure_scan(uint32_t n) {
+        if (sc_mem && n <= sc_n) return MANTRA_OK;
+        n = std::max(n, sc_n);
+        if (sc_mem) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sc_mem); sc_mem = nullptr; }
+        CU(scan_configure(smem_optin));
+        const size_t region = scan_region_bytes(n, &scws);
+        const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 2, free_device_bytes() / 6 / region));
+        if (cudaMalloc(&sc_mem, (size_t)grid * region) != cudaSuccess) { sc_mem = nullptr; return MANTRA_E_NOMEM; }
+        CU(cudaMemsetAsync(sc_mem, 0, (size_t)grid * region, sa));
+        scws.base = sc_mem;
+        scws.stride = region;
+        sc_regions = grid;
+        sc_n = n;
+        invalidate_graph();
+        return MANTRA_OK;
+    }
+
+    // Resident CTAs of k_scan; 0: the bits do not fit.
+    int scan_grid(int nt, uint32_t nsm) {
+        const size_t smem = scan_smem_bytes(nt, nsm);
+        if (smem > smem_optin) return 0;
+        const uint64_t key = ((uint64_t)nsm << 1) | (nt == 1024 ? 1u : 0u);
+        auto it = sc_occ.find(key);
+        if (it == sc_occ.end()) {
+            int per = 0;
+            if (scan_blocks_per_sm(nt, smem, &per) != cudaSuccess) per = 0;
+            it = sc_occ.emplace(key, per).first;
+        }
+        return std::min(sc_regions, it->second * num_sms);
+    }
+
     // The tick as stream work: tables up, slots cleared, both search
     // families on two streams, the round reduction, slots down.
     int enqueue(bool wide) {
         CU(cudaMemcpyAsync(tab_d, tab_h, tab_bytes, cudaMemcpyHostToDevice, sa));
         CU(cudaMemsetAsync(slot_d, 0, (size_t)cap * SLOT_BYTES, sa));
-        if (tick_p || tick_s) {
+        if (tick_p || tick_s || tick_n) {
             CU(cudaEventRecord(ev_fork, sa));
             CU(cudaStreamWaitEvent(sb, ev_fork, 0));
         }
@@ -670,13 +747,20 @@ struct Engine {
                           bfs_grids[shape_of(tick_bfs_nt)][tick_bfs_sm], tick_bfs_sm ? bfs_smem : 0, wide, sa));
         }
         if (tick_b || tick_h) CU(cudaEventRecord(e_b1, sa));
-        if (tick_p || tick_s) CU(cudaEventRecord(e_p0, sb));
+        if (tick_p || tick_s || tick_n) CU(cudaEventRecord(e_p0, sb));
         if (tick_s) {
             SweepWs w = sws;
             w.n_smem = tick_sw_n;
             w.order = tick_sw_order ? sw_order : nullptr;
             CU(launch_sweep((const Task*)(tab_d + o_ts), (const uint64_t*)(tab_d + o_us), hdr + 4, work + 3, w,
                             sweep_grid(tick_sw_n), sb));
+        }
+        if (tick_n) {
+            ScanWs w = scws;
+            w.nt = tick_sc_nt;
+            w.n_smem = tick_sc_n;
+            CU(launch_scan((const Task*)(tab_d + o_tn), (const uint64_t*)(tab_d + o_un), hdr + 5, work + 4, w,
+                           scan_grid(tick_sc_nt, tick_sc_n), sb));
         }
         if (tick_p && tick_cta) {
             PfmCtaWs w = pcws;
@@ -689,7 +773,7 @@ struct Engine {
             CU(launch_pfm((const Task*)(tab_d + o_tp), (const uint64_t*)(tab_d + o_up), hdr + 1, work + 1, pws,
                           pfm_grid, wide, sb));
         }
-        if (tick_p || tick_s) {
+        if (tick_p || tick_s || tick_n) {
             CU(cudaEventRecord(e_p1, sb));
             CU(cudaEventRecord(ev_join, sb));
             CU(cudaStreamWaitEvent(sa, ev_join, 0));
@@ -703,7 +787,7 @@ struct Engine {
     int launch_tick(bool wide) {
         last_tick_graph = false;
         if (wide || !use_graph) return enqueue(wide);
-        const int gk = tick_key();
+        const uint64_t gk = tick_key();
         if (!gexec.count(gk)) {
             cudaGraph_t graph = nullptr;
             CU(cudaStreamBeginCapture(sa, cudaStreamCaptureModeThreadLocal));
@@ -797,10 +881,35 @@ bool pfm_use_cta() {
     return !(env && std::strcmp(env, "lane") == 0);
 }
 
+// Whether the scan (k_scan) takes an item's pfm samples instead of the
+// label-correcting search (k_pfm_cta).  The scan's work is the edges of the window,
+// the search's the out-edges of the vertices reached, so on graphs of bursts (most
+// edges repeat a pair) the search has less to do, and its per-sample arrays are
+// in L2 as long as n is small.  Measured, ms (bursty / uniform times; scan, search):
+//   n = 1,000    231 samples 0.106, 0.122          2,000 samples 0.293, 0.379
+//   n = 5,000     32 0.169, 0.190 / 0.110, 0.212     231 0.288, 0.233 / 0.222, 0.271
+//   n = 20,000    32 0.602, 0.674 / 0.309, 0.637     231 0.973, 0.733 / 0.529, 0.944
+//   n = 50,000    32 1.00, 0.97 / 0.84, 1.17         231 1.89, 1.10 / 1.20, 2.02
+//   n = 100,000   32 1.67, 3.08                      2,000 9.87, 11.2
+//   n = 200,000   32 - / 3.11, 8.07                  1,000 - / 10.5, 38.6
+//   n = 10^6      32 - / 15.2, 47.2                  1,000 - / 55.2, 264
+// so: small graphs and large ones always, the others while each sample has an SM
+// to itself.  (Large rounds of the others are the sweep's.)
+// MANTRA_PFM_KERNEL=scan takes all that can, cta and lane none.
+bool use_scan(const Engine& E, const TickItem& it) {
+    const Job& j = it.job;
+    if (j.opt != MANTRA_PFM || j.ob || j.rtb || j.stats || !it.G->dg.n_scan || it.G->knobs.pfm_search) return false;
+    if (const char* env = std::getenv("MANTRA_PFM_KERNEL")) {
+        if (std::strcmp(env, "lane") == 0 || std::strcmp(env, "cta") == 0) return false;
+        if (std::strcmp(env, "scan") == 0) return true;
+    }
+    return it.G->m <= (1u << 16) || it.G->n > (1u << 16) || j.count <= (uint64_t)E.num_sms;
+}
+
 // Whether the sweep (k_sweep) can take an item's samples.
 bool can_sweep(const TickItem& it) {
     const Job& j = it.job;
-    return j.opt == MANTRA_PFM && !j.ob && !j.rtb && !j.stats && it.G->dg.n_waves > 0;
+    return j.opt == MANTRA_PFM && !j.ob && !j.rtb && !j.stats && it.G->dg.n_waves > 0 && !it.G->knobs.pfm_search;
 }
 
 // Whether a tick's pfm samples take the sweep where they can.  The sweep's time
@@ -825,8 +934,7 @@ bool use_sweep(Engine& E, const std::vector<TickItem>& items) {
     }
     if (!n) return false;
     if (const char* env = std::getenv("MANTRA_PFM_KERNEL")) {
-        if (std::strcmp(env, "lane") == 0 || std::strcmp(env, "cta") == 0) return false;
-        if (std::strcmp(env, "sweep") == 0) return true;
+        return std::strcmp(env, "sweep") == 0;
     }
     int cls = 0;
     const int per = std::max(1, E.sweep_per_sm(Engine::node_step(n, &cls)));
@@ -848,7 +956,9 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     const mantra_graph* gh = nullptr;   // the tick's largest k_hop graph
     bool any_s = false;
     uint32_t sn = 0, smx = 0;
-    uint64_t sunits = 0;
+    uint64_t sunits = 0, nsamples = 0;
+    bool any_n = false;
+    uint32_t nn = 0;
     std::vector<char> sweep(k, 0);
     const bool sweeps = !wide && use_sweep(E, items);
     for (uint32_t x = 0; x < k; ++x) {
@@ -857,6 +967,10 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             sweep[x] = 1;
             any_s = true; sn = std::max(sn, it.G->n); smx = std::max(smx, it.G->m);
             sunits += (it.job.count + 31) / 32;
+        } else if (!wide && use_scan(E, it)) {
+            sweep[x] = 2;
+            any_n = true; nn = std::max(nn, it.G->n);
+            nsamples += it.job.count;
         } else if (it.job.opt == MANTRA_PFM) {
             any_p = true; pn = std::max(pn, it.G->n); plc = std::max(plc, it.G->dg.cbound);
             pz = std::max(pz, it.G->dg.max_vslots);
@@ -873,7 +987,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             dl |= it.job.ob || it.job.rtb;
         }
     }
-    E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p; E.tick_s = any_s;
+    E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p; E.tick_s = any_s; E.tick_n = any_n;
     const bool cta = any_p && !wide && pfm_use_cta();
     if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
     if (any_s) {
@@ -885,6 +999,19 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         if (!E.sweep_grid(E.tick_sw_n)) {
             E.tick_sw_n = E.sw_n;
             E.tick_sw_cls = 255;
+        }
+    }
+    if (any_n) {
+        if ((rc = E.ensure_scan(nn)) != MANTRA_OK) return rc;
+        E.tick_sc_n = Engine::node_step(nn, &E.tick_sc_cls);
+        // CTA size, ms with 512 and 1,024 threads: few samples want each of them fast
+        // (n = 1,000 bursty 231 samples 0.117, 0.106; 2,000 samples 0.293, 0.413), large
+        // graphs have the more edges of a chunk to work on (n = 100,000 2,000 samples
+        // 10.06, 9.87; n = 200,000 11.4, 10.5; n = 10^6 88, 55: one CTA per SM either way).
+        E.tick_sc_nt = nsamples <= 2 * (uint64_t)E.num_sms || nn > (1u << 16) ? 1024 : 512;
+        if (!E.scan_grid(E.tick_sc_nt, E.tick_sc_n)) {       // near the limit: the largest size seen, which fits
+            E.tick_sc_n = E.sc_n;
+            E.tick_sc_cls = 255;
         }
     }
     if (any_b && (rc = E.ensure_bfs(bn, bA, bz, dl)) != MANTRA_OK) return rc;
@@ -973,6 +1100,8 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     u64* work = (u64*)(E.tab_h + E.o_work);
     uint64_t* ub = (uint64_t*)(E.tab_h + E.o_ub);
     uint64_t* up = (uint64_t*)(E.tab_h + E.o_up);
+    uint64_t* un = (uint64_t*)(E.tab_h + E.o_un);
+    Task* tn = (Task*)(E.tab_h + E.o_tn);
     uint64_t* us = (uint64_t*)(E.tab_h + E.o_us);
     Task* tsw = (Task*)(E.tab_h + E.o_ts);
     uint64_t* uh = (uint64_t*)(E.tab_h + E.o_uh);
@@ -981,15 +1110,19 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     Task* tp = (Task*)(E.tab_h + E.o_tp);
     ReduceItem* ri = (ReduceItem*)(E.tab_h + E.o_ri);
     uint32_t* rs = (uint32_t*)(E.tab_h + E.o_rs);
-    uint32_t nb = 0, np = 0, nr = 0, nh = 0, ns = 0;
-    ub[0] = 0; up[0] = 0; uh[0] = 0; us[0] = 0; rs[0] = 0;
+    uint32_t nb = 0, np = 0, nr = 0, nh = 0, ns = 0, nk = 0;
+    ub[0] = 0; up[0] = 0; uh[0] = 0; us[0] = 0; un[0] = 0; rs[0] = 0;
     for (uint32_t x = 0; x < k; ++x) {
         TickItem& it = items[x];
         char* slot = E.slot_d + (size_t)x * SLOT_BYTES;
         it.job.ctr = (u64*)slot;
         it.job.status = (int*)(slot + SLOT_STATUS);
         Task t{it.G->dg, it.job};
-        if (sweep[x]) {
+        if (sweep[x] == 2) {
+            tn[nk] = t;
+            un[nk + 1] = un[nk] + it.job.count;
+            ++nk;
+        } else if (sweep[x]) {
             tsw[ns] = t;
             us[ns + 1] = us[ns] + (it.job.count + 31) / 32;
             ++ns;
@@ -1009,14 +1142,14 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             ++nr;
         }
     }
-    hdr[0] = nb; hdr[1] = np; hdr[2] = nr; hdr[3] = nh; hdr[4] = ns;
-    work[0] = 0; work[1] = 0; work[2] = 0; work[3] = 0;
+    hdr[0] = nb; hdr[1] = np; hdr[2] = nr; hdr[3] = nh; hdr[4] = ns; hdr[5] = nk;
+    work[0] = 0; work[1] = 0; work[2] = 0; work[3] = 0; work[4] = 0;
     if ((rc = E.launch_tick(wide)) != MANTRA_OK) return rc;
     CU(cudaStreamSynchronize(E.sa));
     out->slot.resize(k);
     for (uint32_t x = 0; x < k; ++x) out->slot[x] = E.slot_h + (size_t)x * SLOT_BYTES;
     out->had_bfs = nb + nh > 0;
-    out->had_pfm = np + ns > 0;
+    out->had_pfm = np + ns + nk > 0;
     if (E.last_tick_graph) {
         // a graph tick is timed as a whole: table upload, searches, reduction, readback
         const double t = elapsed_ms(E.e_t0, E.e_t1);
@@ -1029,7 +1162,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     for (uint32_t x = 0; x < k; ++x) {
         const u64* c = (const u64*)out->slot[x];
         if (sweep[x])
-            log_item(items[x], "k_sweep", wide, 32, 0, c, out->pfm_ms);
+            log_item(items[x], sweep[x] == 2 ? "k_scan" : "k_sweep", wide, sweep[x] == 2 ? E.tick_sc_nt : 32, 0, c, out->pfm_ms);
         else if (items[x].job.opt == MANTRA_PFM)
             log_item(items[x], cta ? "k_pfm_cta" : "k_pfm", wide, cta ? E.tick_pc_nt : 32, cta ? E.tick_pc_sm : 0, c,
                      out->pfm_ms);
@@ -1646,6 +1779,7 @@ int mantra_graph_load(const uint32_t* u, const uint32_t* v, const uint32_t* t, u
         rc = E->store.build(u, v, t, m, n, &H);
         if (rc == MANTRA_OK) rc = upload_store(H, G, E->pool, E->sa);
         if (rc == MANTRA_OK) rc = build_waves(G, E->smem_optin, E->pool, E->sa);
+        if (rc == MANTRA_OK) rc = build_chunks(G, E->smem_optin, E->pool, E->sa);
         E->store.trim();
     }
     if (rc != MANTRA_OK) { mantra_graph_free(G); return rc; }
@@ -1692,9 +1826,11 @@ void mantra_graph_free(mantra_graph* g) {
         cudaStreamSynchronize(E->sb);
         E->pool.put(g->dmem, g->b_dmem);
         E->pool.put(g->wmem, g->b_wmem);
+        E->pool.put(g->smem, g->b_smem);
     } else {
         if (g->dmem) cudaFree(g->dmem);
         if (g->wmem) cudaFree(g->wmem);
+        if (g->smem) cudaFree(g->smem);
     }
     delete g;
 }
@@ -1742,10 +1878,12 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
     };
     const Knobs none{};
     Knobs best{};
+    Knobs search{};      // pfm's defaults on the kernel whose knobs are probed
+    search.pfm_search = true;
     auto size_probe = [&](mantra_opt opt) -> int {
         r = r_lo;
         double ms = 0;
-        const int st = probe(opt, none, &ms);
+        const int st = probe(opt, search, &ms);
         if (st != MANTRA_OK) return st;
         const double per = ms > 0 ? ms / (double)r_lo : 0.0;
         r = per > 0 ? (uint64_t)std::min<double>((double)r_hi, std::max<double>((double)r_lo, 100.0 / per)) : r_hi;
@@ -1768,13 +1906,13 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
     // pfm (one CTA per sample): CTA shape x arrival-state placement
     if ((rc = size_probe(MANTRA_PFM)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->pfm_probe_samples = r;
-    if ((rc = probe(MANTRA_PFM, none, &out->pfm_default_ms)) != MANTRA_OK) { g->knobs = none; return rc; }
+    if ((rc = probe(MANTRA_PFM, search, &out->pfm_default_ms)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->pfm_ms = 1e300;
     for (int nt : {256, 512})
         for (int sm = 0; sm < 4; ++sm) {
             if (!E->pc_grids[nt == 256 ? 0 : 1][sm]) continue;
             if (sm == 3 && g->dg.max_vslots > PFM_W16_MAX_VSLOTS) continue;
-            Knobs k = none;
+            Knobs k = search;
             k.pfm_nt = nt; k.pfm_mode = sm;
             double ms = 0;
             if ((rc = probe(MANTRA_PFM, k, &ms)) != MANTRA_OK) { g->knobs = none; return rc; }

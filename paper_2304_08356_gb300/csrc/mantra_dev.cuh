@@ -74,6 +74,9 @@ struct DevGraph {
     const uint32_t* dir_t;       // dir_n bucket times, ascending, the first 0
     uint32_t dir_n;              // buckets of the times (at most 32)
     // the stream cut into waves of at most 32 independent edges (k_sweep.cu; none: n_waves = 0)
+    uint32_t n_scan;             // chunks of whole time steps of the stream (k_scan.cu; none: 0)
+    const uint32_t* scan_ptr;    // n_scan + 1: their first stream edges
+    const uint32_t* st_slot;     // per stream edge: the head's slot
     uint32_t n_waves;            // a multiple of WAVE_BATCH
     const uint2* wave_uv;        // 32 per wave: u, v (padding: n, n)
     const uint2* wave_at;        // 32 per wave: the head's slot, t
@@ -88,6 +91,10 @@ struct DevGraph {
 // them; an edge's head slot has several in-edges.
 constexpr uint32_t WAVE_CUT = 128, WAVE_STEP = 512, WAVE_BATCH = 8;
 constexpr uint32_t WAVE_BIG = 1u, WAVE_LAST = 2u, WAVE_SEVERAL = 4u;
+
+// Stream edges between the cuts of k_scan's chunks: a chunk takes this many or a
+// little more, up to 2,048, as it ends with its last edge's time step.
+constexpr uint32_t SCAN_CHUNK = 1536;
 
 // The waves' arrays while they are filled (see DevGraph).
 struct WaveArrays {
@@ -800,6 +807,15 @@ struct HopWs {
     uint32_t n_smem;     // nodes whose next-level arrivals are in dynamic shared memory (0: in the region)
 };
 
+// Per-CTA scratch of the pfm scan of the stream.
+struct ScanWs {
+    char* base;          // CTA b uses base + b * stride
+    size_t stride;
+    size_t o_arr, o_path, o_pathe, o_cv, o_co, o_ck, o_sig, o_mk;
+    uint32_t n_smem;     // nodes of the shared-memory bits
+    int nt;              // threads per CTA (512 or 1024)
+};
+
 // Per-warp scratch of the pfm sweep over the stream (one region per CTA).
 struct SweepWs {
     char* base;          // CTA b uses base + b * stride
@@ -856,6 +872,14 @@ cudaError_t launch_hop(const Task* tasks, const uint64_t* unit_start, const uint
 struct DirTimes { uint32_t t[32]; };
 cudaError_t launch_edge_maps(const DevGraph& g, const DirTimes& dt, uint2* out_vn, uint32_t* in_out, uint32_t* out_pend,
                              uint2* dir, uint32_t* dir_t, cudaStream_t st);
+size_t scan_region_bytes(uint32_t n, ScanWs* ws);
+size_t scan_smem_bytes(int nt, uint32_t n);
+cudaError_t scan_configure(size_t smem);
+cudaError_t scan_blocks_per_sm(int nt, size_t smem, int* out);
+cudaError_t launch_scan(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
+                        const ScanWs& ws, int grid, cudaStream_t st);
+// Fills st_slot (m), scan_ptr (ceil(m / SCAN_CHUNK) + 1) and *big (a chunk would exceed 2,048 edges: no scan).
+cudaError_t launch_scan_maps(const DevGraph& g, uint32_t* st_slot, uint32_t* ptr, uint32_t* big, cudaStream_t st);
 size_t sweep_region_bytes(uint32_t n, uint32_t m, SweepWs* ws);
 size_t sweep_smem_bytes(uint32_t n);
 size_t sweep_static_smem();
