@@ -158,7 +158,8 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-KSRC = {"k_hop": "k_hop.cu", "k_bfs": "k_bfs.cu", "k_pfm_cta": "k_pfm_cta.cu", "k_pfm": "k_pfm.cu"}
+KSRC = {"k_hop": "k_hop.cu", "k_bfs": "k_bfs.cu", "k_pfm_cta": "k_pfm_cta.cu", "k_pfm": "k_pfm.cu",
+        "k_sweep": "k_sweep.cu", "k_scan": "k_scan.cu"}
 
 
 def kernel_source_digest(kernel: str):
@@ -279,13 +280,15 @@ def kernel_rooflines(info, opt, peak, ms=None):
     ms = info["kernel_ms"] if ms is None else ms
     out = {}
     if opt == "pfm":
-        own = 12 * info["edges_expanded"] + 24 * info["sigma_adds"]
-        out["k_pfm_cta"] = {"achieved": info["alg_bytes"] / (ms / 1e3) / 1e9,
-                            "achieved_own_model": own / (ms / 1e3) / 1e9,
-                            "alg_bytes": info["alg_bytes"], "own_model_bytes": own, "ms": ms,
-                            "launches": info["search_launches"]}
-        out["k_pfm_cta"]["frac"] = out["k_pfm_cta"]["achieved"] / peak
-        out["k_pfm_cta"]["frac_own_model"] = out["k_pfm_cta"]["achieved_own_model"] / peak
+        k = "k_scan"            # the large graph's kernel; it expands no out-edges
+        out[k] = {"achieved": info["alg_bytes"] / (ms / 1e3) / 1e9, "alg_bytes": info["alg_bytes"], "ms": ms,
+                  "launches": info["search_launches"]}
+        if info["edges_expanded"]:
+            own = 12 * info["edges_expanded"] + 24 * info["sigma_adds"]
+            out["k_pfm_cta"] = dict(out.pop(k), achieved_own_model=own / (ms / 1e3) / 1e9, own_model_bytes=own)
+            k = "k_pfm_cta"
+            out[k]["frac_own_model"] = out[k]["achieved_own_model"] / peak
+        out[k]["frac"] = out[k]["achieved"] / peak
     else:
         out["k_hop"] = {"achieved": info["alg_bytes"] / (ms / 1e3) / 1e9, "alg_bytes": info["alg_bytes"], "ms": ms,
                         "launches": info["search_launches"]}
@@ -640,7 +643,8 @@ def main():
                             "kernel_ms": {o: r[2]["kernel_ms"] for o, r in zip(OPTS, res)}}
 
     # dominant kernel: search time per optimality family (sequential pass)
-    pfm_kernel = "k_pfm" if os.environ.get("MANTRA_PFM_KERNEL") == "lane" else "k_pfm_cta"
+    # (a pfm run's rounds are the sweep's; its bootstrap and first rounds are k_pfm_cta's)
+    pfm_kernel = {"lane": "k_pfm", "cta": "k_pfm_cta"}.get(os.environ.get("MANTRA_PFM_KERNEL"), "k_sweep")
     fam = {k: tuple(o for o in v_ if o in OPTS) for k, v_ in {"k_hop": ("sh", "sfm"), pfm_kernel: ("pfm",)}.items()}
     fam = {k: v_ for k, v_ in fam.items() if v_}
     kms = {k: sum(st[o]["kernel_ms"] for st in seq_infos for o in os_) for k, os_ in fam.items()}
