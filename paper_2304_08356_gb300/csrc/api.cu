@@ -228,7 +228,9 @@ int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
     const bool force = env && std::strcmp(env, "scan") == 0;
-    if (m == 0 || !(force || few_choices(G)) || scan_smem_bytes(1024, G->n) > smem_optin) return MANTRA_OK;
+    // (a chunk's last index must not wrap)
+    if (m == 0 || m > 0xFFFF0000u || !(force || few_choices(G)) ||
+        scan_smem_bytes(1024, G->n) > smem_optin) return MANTRA_OK;
     const size_t nc = ((size_t)m + SCAN_CHUNK - 1) / SCAN_CHUNK;
     G->b_smem = al256((size_t)m * 4) + al256((nc + 1) * 4) + 256;
     G->smem = pool.get(G->b_smem);
@@ -336,6 +338,7 @@ struct Engine {
     uint32_t tick_sc_n = 0;
     std::map<uint64_t, int> sc_occ;        // (threads, shared nodes) -> CTAs per SM
     bool tick_n = false;
+    bool search_only = false;              // this tick: no room for k_sweep's or k_scan's workspace
     bool tick_b = false, tick_h = false, tick_p = false;   // kernel families with samples in the current tick
     char* pfm_mem = nullptr; PfmWs pws{}; int pfm_grid = 0; uint32_t pfm_n = 0, pfm_lcap = 0; uint64_t pfm_warps = 0;
     // pfm, one CTA per sample: shapes 0 = 256, 1 = 512 threads; modes 0 = state
@@ -960,14 +963,14 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     bool any_n = false;
     uint32_t nn = 0;
     std::vector<char> sweep(k, 0);
-    const bool sweeps = !wide && use_sweep(E, items);
+    const bool sweeps = !wide && !E.search_only && use_sweep(E, items);
     for (uint32_t x = 0; x < k; ++x) {
         const TickItem& it = items[x];
         if (sweeps && can_sweep(it)) {
             sweep[x] = 1;
             any_s = true; sn = std::max(sn, it.G->n); smx = std::max(smx, it.G->m);
             sunits += (it.job.count + 31) / 32;
-        } else if (!wide && use_scan(E, it)) {
+        } else if (!wide && !E.search_only && use_scan(E, it)) {
             sweep[x] = 2;
             any_n = true; nn = std::max(nn, it.G->n);
             nsamples += it.job.count;
@@ -990,9 +993,20 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p; E.tick_s = any_s; E.tick_n = any_n;
     const bool cta = any_p && !wide && pfm_use_cta();
     if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
+    // a device too full for the workspaces of the passes over the stream runs the
+    // search, whose workspace may be there already
+    rc = any_s ? E.ensure_sweep(sn, smx) : MANTRA_OK;
+    if (rc == MANTRA_OK && any_s) rc = E.ensure_sweep_order(sunits);
+    if (rc == MANTRA_OK && any_n) rc = E.ensure_scan(nn);
+    if (rc == MANTRA_E_NOMEM) {
+        (void)cudaGetLastError();
+        E.search_only = true;
+        rc = run_tick(E, items, wide, out);
+        E.search_only = false;
+        return rc;
+    }
+    if (rc != MANTRA_OK) return rc;
     if (any_s) {
-        if ((rc = E.ensure_sweep(sn, smx)) != MANTRA_OK) return rc;
-        if ((rc = E.ensure_sweep_order(sunits)) != MANTRA_OK) return rc;
         E.tick_sw_n = Engine::node_step(sn, &E.tick_sw_cls);
         // near the limit the step may not fit: the graphs' own size then (a graph with
         // waves fits), captured as the last step
@@ -1002,7 +1016,6 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         }
     }
     if (any_n) {
-        if ((rc = E.ensure_scan(nn)) != MANTRA_OK) return rc;
         E.tick_sc_n = Engine::node_step(nn, &E.tick_sc_cls);
         // CTA size, ms with 512 and 1,024 threads: few samples want each of them fast
         // (n = 1,000 bursty 231 samples 0.117, 0.106; 2,000 samples 0.293, 0.413), large
