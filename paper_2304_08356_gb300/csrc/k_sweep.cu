@@ -31,6 +31,7 @@
 // 4 n bytes a warp.  42,000 samples of the bursty 20,000-node graph take 9.1
 // ms; a search per sample (k_pfm_cta) takes 33.4 ms.
 #include "mantra_dev.cuh"
+#include "waves.h"
 
 #include <algorithm>
 #include <mutex>
@@ -664,35 +665,50 @@ __global__ void k_wave_deps(DevGraph g, const uint32_t* slot, const uint32_t* sl
     dep[i] = d;
 }
 
-// Cuts the stream into waves: thread x takes the time steps that begin in
-// [x CUT, (x + 1) CUT) and extends a wave by whole steps while it has at most
-// 32 edges and none depends on an edge of the wave; a step of more edges gets
-// waves of its own.  start: the waves' first edges, from x CUT (a wave has at
-// least one edge, so the parts' places do not overlap); count[x]; *big: a step
-// has more than WAVE_STEP waves.
-__global__ void k_wave_cut(DevGraph g, const uint32_t* dep, uint32_t* start, uint32_t* count, uint32_t* big) {
+// Cuts the stream into waves (wave_cut_part), a thread per part.  A wave is noted
+// at its own first edge: marks[i] = 1 (zeroed before), which no other thread
+// writes.  *big: a step has more than WAVE_STEP waves.
+__global__ void k_wave_cut(DevGraph g, const uint32_t* dep, unsigned char* marks, uint32_t* big) {
     const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint64_t lo = (uint64_t)x * WAVE_CUT;
-    if (lo >= g.m) return;
-    const uint32_t hi = (uint32_t)min(lo + (uint64_t)WAVE_CUT, (uint64_t)g.m);
-    uint32_t i = (uint32_t)lo, c = 0;
-    while (i > 0 && i < hi && g.st_t[i] == g.st_t[i - 1]) ++i;       // a step that began earlier
-    uint32_t s = i;
-    bool open = false;
-    while (i < hi) {
-        const uint32_t tm = g.st_t[i];                                // the step [i, e)
-        uint32_t e = i, d = 0;
-        while (e < g.m && g.st_t[e] == tm) { d = max(d, dep[e]); ++e; }
-        if (e - i > 32u) {                                            // several waves for the step
-            if (e - i > 32u * WAVE_STEP) { atomicMax(big, 1u); break; }
-            for (uint32_t y = i; y < e; y += 32u) start[lo + c++] = y;
-            open = false;
-        } else if (!open || d > s || e - s > 32u) {
-            s = i; open = true; start[lo + c++] = s;
-        }
-        i = e;
+    if (!wave_cut_part(g.st_t, dep, g.m, x, [&](uint32_t i) { marks[i] = 1; })) atomicMax(big, 1u);
+}
+
+// The marks of a part: four edges per lane of a warp; the lane's number of marks
+// and, in *before, those of the lanes before it.
+__device__ __forceinline__ uint32_t wave_marks(const unsigned char* marks, uint32_t x, uint32_t* word, uint32_t* before) {
+    static_assert(WAVE_CUT == 128, "a warp takes a part, four edges a lane");
+    const uint32_t lane = threadIdx.x & 31;
+    *word = reinterpret_cast<const uint32_t*>(marks)[(size_t)x * 32u + lane];
+    const uint32_t c = __popc(*word);
+    uint32_t incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
+        if (lane >= (uint32_t)o) incl += y;
     }
-    count[x] = c;
+    *before = incl - c;
+    return c;
+}
+
+// count[x]: marks of part x.
+__global__ void k_wave_count(const unsigned char* marks, uint32_t nb, uint32_t* count) {
+    const uint32_t x = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    if (x >= nb) return;
+    uint32_t word, before;
+    const uint32_t c = wave_marks(marks, x, &word, &before);
+    if ((threadIdx.x & 31) == 31) count[x] = before + c;
+}
+
+// first[w]: the first edge of wave w (base: the exclusive sums of count).
+__global__ void k_wave_first(const unsigned char* marks, uint32_t nb, const uint32_t* base, uint32_t* first) {
+    const uint32_t x = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
+    if (x >= nb) return;
+    uint32_t word, before;
+    wave_marks(marks, x, &word, &before);
+    uint32_t* f = first + base[x] + before;
+#pragma unroll
+    for (uint32_t y = 0; y < 4; ++y)
+        if ((word >> (8u * y)) & 1u) *f++ = x * WAVE_CUT + (threadIdx.x & 31) * 4u + y;
 }
 
 // Exclusive sums of count (one CTA); *total.
@@ -715,21 +731,11 @@ __global__ void __launch_bounds__(1024) k_wave_sum(uint32_t* count, uint32_t nb,
 
 // The waves' edges, 32 places each (padding: u = v = n), up to a multiple of
 // WAVE_BATCH waves; a wave ends where the next begins.
-__global__ void k_wave_fill(DevGraph g, const uint32_t* slot, const uint32_t* start, const uint32_t* base, uint32_t nb,
-                            uint32_t total, WaveArrays wa) {
+__global__ void k_wave_fill(DevGraph g, const uint32_t* slot, const uint32_t* first, uint32_t total, WaveArrays wa) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t w = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (w >= wa.n_waves) return;
-    auto first = [&](uint32_t y) -> uint32_t {                        // first edge of wave y
-        if (y >= total) return g.m;
-        uint32_t lo = 0, hi = nb;                                     // the last part x with base[x] <= y
-        while (hi - lo > 1) {
-            const uint32_t mid = (lo + hi) >> 1;
-            if (base[mid] <= y) lo = mid; else hi = mid;
-        }
-        return start[(size_t)lo * WAVE_CUT + (y - base[lo])];
-    };
-    const uint32_t i0 = first(w), i1 = w + 1 < total ? first(w + 1) : g.m, i = i0 + lane;
+    const uint32_t i0 = w < total ? first[w] : g.m, i1 = w + 1 < total ? first[w + 1] : g.m, i = i0 + lane;
     uint2 uv = make_uint2(g.n, g.n), at = make_uint2(0u, 0u);
     uint32_t fl = 0;
     if (i < i1) {
@@ -737,13 +743,10 @@ __global__ void k_wave_fill(DevGraph g, const uint32_t* slot, const uint32_t* st
         uv = make_uint2(g.st_u[i], g.st_v[i]);
         at = make_uint2(a, tm);
         if (g.slot_in[a + 1] - g.slot_in[a] > 1u) fl = WAVE_SEVERAL;
-        // a wave that shares its time with a neighbour is part of a step of several waves
-        const bool more = i1 < g.m && g.st_t[i1] == tm;
-        if (more || (i0 > 0 && g.st_t[i0 - 1] == tm && g.st_t[i1 - 1] == tm)) fl |= WAVE_BIG | (more ? 0u : WAVE_LAST);
     }
     wa.uv[(size_t)w * 32u + lane] = uv;
     wa.at[(size_t)w * 32u + lane] = at;
-    fl = __reduce_or_sync(0xFFFFFFFFu, fl);
+    fl = __reduce_or_sync(0xFFFFFFFFu, fl) | wave_step_flags(g.st_t, g.m, i0, i1);
     if (lane == 0) {
         wa.fl[w] = fl;
         wa.t[w] = g.st_t[(i1 ? i1 : 1u) - 1u];
@@ -752,25 +755,29 @@ __global__ void k_wave_fill(DevGraph g, const uint32_t* slot, const uint32_t* st
     }
 }
 
-// Waves of g, first part: the cut.  tmp: wave_tmp_bytes(m, A); the number of
-// waves and the oversize flag end in its first two words.
+// Waves of g, first part: the cut.  tmp (wave_tmp_bytes(m, A)): the number of waves
+// and the oversize flag in its first two words | marks | slot | dep, then first |
+// last | count.
 size_t wave_tmp_bytes(uint32_t m, uint32_t A) {
     const size_t nb = ((size_t)m + WAVE_CUT - 1) / WAVE_CUT;
-    return 256 + ((size_t)m * 3 + A + nb + 64) * 4;
+    return 256 + nb * WAVE_CUT + ((size_t)m * 2 + A + nb + 64) * 4;
 }
 
 cudaError_t launch_wave_cut(const DevGraph& g, char* tmp, cudaStream_t st) {
     const uint32_t nb = (g.m + WAVE_CUT - 1) / WAVE_CUT;
     uint32_t* head = reinterpret_cast<uint32_t*>(tmp);
-    uint32_t* slot = reinterpret_cast<uint32_t*>(tmp + 256);
-    uint32_t *dep = slot + g.m, *start = dep + g.m, *last = start + g.m, *count = last + g.A;
-    cudaError_t e = cudaMemsetAsync(head, 0, 8, st);
+    unsigned char* marks = reinterpret_cast<unsigned char*>(tmp + 256);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(tmp + 256 + (size_t)nb * WAVE_CUT);
+    uint32_t *dep = slot + g.m, *last = dep + g.m, *count = last + g.A;
+    cudaError_t e = cudaMemsetAsync(tmp, 0, 256 + (size_t)nb * WAVE_CUT, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(last, 0, (size_t)g.A * 4, st);
     if (e != cudaSuccess) return e;
     k_wave_slots<<<(g.m + 255) / 256, 256, 0, st>>>(g, slot, last);
     k_wave_deps<<<(g.m + 255) / 256, 256, 0, st>>>(g, slot, last, dep);
-    k_wave_cut<<<(nb + 31) / 32, 32, 0, st>>>(g, dep, start, count, head + 1);
+    k_wave_cut<<<(nb + 31) / 32, 32, 0, st>>>(g, dep, marks, head + 1);
+    k_wave_count<<<(nb + 7) / 8, 256, 0, st>>>(marks, nb, count);
     k_wave_sum<<<1, 1024, 0, st>>>(count, nb, head);
+    k_wave_first<<<(nb + 7) / 8, 256, 0, st>>>(marks, nb, count, dep);
     return cudaGetLastError();
 }
 
@@ -781,9 +788,8 @@ size_t wave_bytes(uint32_t total) {
 
 // Second part: the waves' arrays, laid out in mem (wave_bytes(total)), filled.
 cudaError_t launch_wave_fill(DevGraph* g, char* tmp, uint32_t total, char* mem, cudaStream_t st) {
-    const uint32_t nb = (g->m + WAVE_CUT - 1) / WAVE_CUT;
-    uint32_t* slot = reinterpret_cast<uint32_t*>(tmp + 256);
-    uint32_t *start = slot + 2 * (size_t)g->m, *count = start + g->m + g->A;
+    const size_t nb = ((size_t)g->m + WAVE_CUT - 1) / WAVE_CUT;
+    const uint32_t* slot = reinterpret_cast<const uint32_t*>(tmp + 256 + nb * WAVE_CUT);
     WaveArrays wa;
     wa.n_waves = (total + WAVE_BATCH - 1) / WAVE_BATCH * WAVE_BATCH;
     wa.uv = reinterpret_cast<uint2*>(mem);
@@ -793,7 +799,7 @@ cudaError_t launch_wave_fill(DevGraph* g, char* tmp, uint32_t total, char* mem, 
     wa.fl = wa.t + wa.n_waves;
     cudaError_t e = cudaMemsetAsync(wa.info, 0, wa.n_waves / WAVE_BATCH * sizeof(uint2), st);
     if (e != cudaSuccess) return e;
-    k_wave_fill<<<(wa.n_waves + 7) / 8, 256, 0, st>>>(*g, slot, start, count, nb, total, wa);
+    k_wave_fill<<<(wa.n_waves + 7) / 8, 256, 0, st>>>(*g, slot, slot + g->m, total, wa);
     g->n_waves = wa.n_waves;
     g->wave_uv = wa.uv; g->wave_at = wa.at; g->wave_info = wa.info; g->wave_t = wa.t; g->wave_fl = wa.fl;
     return cudaGetLastError();

@@ -85,13 +85,6 @@ struct DevGraph {
     const uint32_t* wave_fl;     // per wave: WAVE_BIG, WAVE_LAST, WAVE_SEVERAL
 };
 
-// Stream edges per part of the wave cut (a thread each: 512 made a load of 125,000
-// edges 0.25 ms longer, 128 a sweep 2 % longer); waves of one time step at most; waves
-// per batch.  Flags of a wave: part of a time step of several waves, the last of
-// them; an edge's head slot has several in-edges.
-constexpr uint32_t WAVE_CUT = 128, WAVE_STEP = 512, WAVE_BATCH = 8;
-constexpr uint32_t WAVE_BIG = 1u, WAVE_LAST = 2u, WAVE_SEVERAL = 4u;
-
 // Stream edges between the cuts of k_scan's chunks: a chunk takes this many or a
 // little more, up to 2,048, as it ends with its last edge's time step.
 constexpr uint32_t SCAN_CHUNK = 1536;

@@ -1,0 +1,50 @@
+"""pfm on streams whose waves are hard to cut (csrc/waves.h, csrc/k_sweep.cu): a
+hub with a run of single contacts and then a time step of several waves, at every
+place of a part of the cut.  Hits, estimates and work counters equal the oracle's,
+and edges_expanded (0 unless the label-correcting search ran) shows that the sweep
+ran."""
+import numpy as np
+import pytest
+
+from oracle import oracle as O
+from test_gpu_sweep import COUNTERS
+from test_wave_cut import PART, hub_stream
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    from paper_2304_08356_gb300 import build as B
+    B.build()
+    from paper_2304_08356_gb300 import mantra
+    return mantra
+
+
+def equal(M, tri, n, r, swept=True):
+    g, o = M.Graph(*tri, n=n), O.Graph(*tri, n=n)
+    _, hits, info = g.estimate(2, 0.05, 0.1, 3, fixed_r=r)
+    _, ohits, oinfo = o.estimate(2, 0.05, 0.1, 3, fixed_r=r)
+    assert np.array_equal(hits, ohits)
+    for k in COUNTERS:
+        assert info[k] == oinfo[k], k
+    assert (info["edges_expanded"] == 0) == swept
+    g.free()
+
+
+@pytest.mark.parametrize("before,step,after,periods", [(127, 33, 160, 60), (150, 40, 177, 60), (300, 100, 301, 40)])
+def test_hub_then_broadcast(M, monkeypatch, before, step, after, periods):
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    equal(M, hub_stream(before, step, after, periods), 1000, 600)
+
+
+@pytest.mark.parametrize("lead", range(PART - 4, PART + 1))
+def test_step_at_the_end_of_a_part(M, monkeypatch, lead):
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    equal(M, hub_stream(lead, 40, 300, 1, n=60), 60, 600)
+
+
+def test_hub_then_broadcast_by_default(M, monkeypatch):
+    """More than 2^16 edges and samples enough that the rules choose the sweep."""
+    monkeypatch.delenv("MANTRA_PFM_KERNEL", raising=False)
+    equal(M, hub_stream(127, 33, 160, 300), 1000, 40000)
