@@ -157,6 +157,7 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
         auto settle = [&](uint32_t log0) {
             const unsigned hit = __ballot_sync(FULL, (act & bit) && (R[z] & bit));
             if (!hit) return;
+            __syncwarp();                                   // (a vote does not order the lanes' log records)
             for (uint32_t p0 = log0; p0 < nlog; p0 += 32) {
                 const uint32_t p = p0 + lane;
                 const uint4 r = p < nlog ? log[p] : make_uint4(n, 0u, 0u, 0u);

@@ -1,6 +1,6 @@
 """pfm on streams whose waves are hard to cut (csrc/waves.h, csrc/k_sweep.cu): a
 hub with a run of single contacts and then a time step of several waves, at every
-place of a part of the cut.  Hits, estimates and work counters equal the oracle's,
+place of a part of the cut, and arrivals in every wave of a batch.  Hits, estimates and work counters equal the oracle's,
 and edges_expanded (0 unless the label-correcting search ran) shows that the sweep
 ran."""
 import numpy as np
@@ -48,3 +48,17 @@ def test_hub_then_broadcast_by_default(M, monkeypatch):
     """More than 2^16 edges and samples enough that the rules choose the sweep."""
     monkeypatch.delenv("MANTRA_PFM_KERNEL", raising=False)
     equal(M, hub_stream(127, 33, 160, 300), 1000, 40000)
+
+
+def test_arrival_in_every_wave_of_a_batch(M, monkeypatch):
+    """A chain has a wave per edge: with all pairs drawn, z is reached in the first
+    to the last wave of a batch of eight, where the sample's last time is read back
+    from the records just written."""
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    c = np.arange(40)
+    tri = tuple(x.astype(np.uint32) for x in (c, c + 1, 3 * c + 5))
+    equal(M, tri, 41, 6000)
+    g, o = M.Graph(*tri, n=41), O.Graph(*tri, n=41)
+    got = g.sample_paths(2, 8, 0, 3000, cap=42)
+    assert got == o.samples(2, 8, 0, 3000, cap=42)
+    g.free()
