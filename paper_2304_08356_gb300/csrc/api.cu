@@ -7,6 +7,7 @@
 // include/mantra.h.
 #include "mantra.h"
 #include "mantra_dev.cuh"
+#include "waves.h"
 #include "store.h"
 
 #include <algorithm>
@@ -193,6 +194,7 @@ bool few_choices(const mantra_graph* G) { return (uint64_t)G->A * 100 >= (uint64
 // under 2^16 edges: k_pfm_cta takes 0.1 us a sample there, and the cut would be
 // a tenth of the load.  Nor graphs in which ways back have
 // choices (few_choices).  MANTRA_PFM_KERNEL=sweep at the load lifts the last three.
+// Nor streams of more waves than a 32-bit place can name (waves_indexable).
 int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
@@ -207,7 +209,7 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
         cudaMemcpyAsync(head, tmp, sizeof head, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
         rc = MANTRA_E_CUDA;
-    if (rc == MANTRA_OK && head[1] == 0 && (force || (uint64_t)head[0] * 2 <= (uint64_t)m)) {
+    if (rc == MANTRA_OK && head[1] == 0 && waves_indexable(head[0]) && (force || (uint64_t)head[0] * 2 <= (uint64_t)m)) {
         G->b_wmem = wave_bytes(head[0]);
         G->wmem = pool.get(G->b_wmem);
         if (!G->wmem) {

@@ -59,4 +59,10 @@ __host__ __device__ inline uint32_t wave_step_flags(const uint32_t* t, uint32_t 
     return more ? WAVE_BIG : (i0 > 0 && t[i0 - 1] == tm ? WAVE_BIG | WAVE_LAST : 0u);
 }
 
+// Whether a stream of that many waves can be swept: a record of the log names
+// its edge by its place in the waves (32 a wave, whole batches) in 32 bits.
+__host__ __device__ inline bool waves_indexable(uint64_t waves) {
+    return (waves + WAVE_BATCH - 1) / WAVE_BATCH * WAVE_BATCH * 32u <= (uint64_t)1 << 32;
+}
+
 }  // namespace mantra

@@ -1,8 +1,8 @@
 """pfm on streams whose waves are hard to cut (csrc/waves.h, csrc/k_sweep.cu): a
 hub with a run of single contacts and then a time step of several waves, at every
-place of a part of the cut, and arrivals in every wave of a batch.  Hits, estimates and work counters equal the oracle's,
-and edges_expanded (0 unless the label-correcting search ran) shows that the sweep
-ran."""
+place of a part of the cut, and arrivals in every wave of a batch.  Hits, estimates
+and work counters equal the oracle's, and edges_expanded (0 unless the
+label-correcting search ran) shows that the sweep ran."""
 import numpy as np
 import pytest
 

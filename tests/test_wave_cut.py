@@ -127,3 +127,11 @@ def test_longest_step(driver, tmp_path, edges):
     assert fit == (edges <= 32 * STEP)
     if fit:
         assert marks == 1 and first == [0] + list(range(1, 1 + edges, 32)) + [1 + edges]
+
+
+@pytest.mark.parametrize("waves", [0, 1, (1 << 27) - 8, (1 << 27) - 7, 1 << 27, (1 << 27) + 1, 1 << 31, (1 << 32) - 1])
+def test_places_fit_in_32_bits(driver, waves):
+    """A place is 32 * wave + lane; the last one of the last batch must not wrap."""
+    last = (waves + 7) // 8 * 8 * 32 - 1
+    r = subprocess.run([driver, "--indexable", str(waves)], capture_output=True, text=True, check=True)
+    assert int(r.stdout) == (1 if last < 1 << 32 else 0)

@@ -2,15 +2,21 @@
 // GPU.  Reads uint64 m, then t[m] and dep[m] as uint32; runs every part of the
 // cut, the last part first, and writes as uint32: 1 if all steps fit, the largest
 // number of marks on one edge, the number of waves, then their first edges and
-// their step flags.
+// their step flags.  With --indexable N it prints whether N waves can be swept.
 #include "waves.h"
 
 #include <algorithm>
 #include <cstdio>
+#include <cstdlib>
+#include <cstring>
 #include <vector>
 
 int main(int argc, char** argv) {
     if (argc != 3) return 2;
+    if (!std::strcmp(argv[1], "--indexable")) {
+        std::printf("%d\n", mantra::waves_indexable(std::strtoull(argv[2], nullptr, 10)) ? 1 : 0);
+        return 0;
+    }
     FILE* f = std::fopen(argv[1], "rb");
     if (!f) return 2;
     uint64_t m = 0;
