@@ -7,8 +7,9 @@
 // include/mantra.h.
 #include "mantra.h"
 #include "mantra_dev.cuh"
-#include "waves.h"
+#include "devmem.h"
 #include "store.h"
+#include "waves.h"
 
 #include <algorithm>
 #include <chrono>
@@ -78,44 +79,21 @@ double now_s() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
 }
 
-// ---------------------------------------------------------------------------
-// Device memory pool: blocks kept by exact (256-rounded) size and reused by
-// later problems and graphs; at most kPoolCacheBytes stay cached.
-// ---------------------------------------------------------------------------
+// Device memory (devmem.h) and page-locked host memory.
+struct CudaMemory {
+    static bool alloc(void** p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; }
+    static void free(void* p) { cudaFree(p); }
+    static void clear() { (void)cudaGetLastError(); }
+};
+struct PinnedMemory {
+    static bool alloc(void** p, size_t bytes) { return cudaMallocHost(p, bytes) == cudaSuccess; }
+    static void free(void* p) { cudaFreeHost(p); }
+    static void clear() { (void)cudaGetLastError(); }
+};
+
 constexpr size_t kPoolCacheBytes = (size_t)8 << 30;
 
-struct DevPool {
-    std::multimap<size_t, void*> free_blocks;
-    size_t cached = 0;
-    void* get(size_t bytes) {
-        bytes = al256(std::max<size_t>(bytes, 256));
-        auto it = free_blocks.find(bytes);
-        if (it != free_blocks.end()) {
-            void* p = it->second;
-            free_blocks.erase(it);
-            cached -= bytes;
-            return p;
-        }
-        void* p = nullptr;
-        if (cudaMalloc(&p, bytes) != cudaSuccess) {
-            release_all();
-            if (cudaMalloc(&p, bytes) != cudaSuccess) return nullptr;
-        }
-        return p;
-    }
-    void put(void* p, size_t bytes) {
-        if (!p) return;
-        bytes = al256(std::max<size_t>(bytes, 256));
-        if (cached + bytes > kPoolCacheBytes) { cudaFree(p); return; }
-        free_blocks.emplace(bytes, p);
-        cached += bytes;
-    }
-    void release_all() {
-        for (auto& kv : free_blocks) cudaFree(kv.second);
-        free_blocks.clear();
-        cached = 0;
-    }
-};
+using DevPool = MemoryPool<CudaMemory>;
 
 // ---------------------------------------------------------------------------
 // Temporal-edge store (paper Sec. 3: the temporal graph; the paper's own code
@@ -360,7 +338,7 @@ struct Engine {
     // captured ticks, by launch configuration (tick_key)
     std::map<uint64_t, cudaGraphExec_t> gexec;
     bool use_graph = true;
-    DevPool pool;
+    DevPool pool{kPoolCacheBytes};
 
     int init(int dev) {
         device = dev;
@@ -420,7 +398,7 @@ struct Engine {
     // Table block layout: header | work counters | unit starts and tasks (bfs, pfm,
     // hop, sweep, scan) | reduction items | reduction row starts.
     int ensure_tables(uint32_t need) {
-        if (tab_h && need <= cap) return MANTRA_OK;
+        if (tab_h && tab_d && slot_h && slot_d && need <= cap) return MANTRA_OK;
         uint32_t nc = std::max<uint32_t>(64, cap);
         while (nc < need) nc *= 2;
         if (tab_h) { cudaFreeHost(tab_h); tab_h = nullptr; }
@@ -443,10 +421,10 @@ struct Engine {
         o_ri = o;   o = al256(o + (size_t)nc * sizeof(ReduceItem));
         o_rs = o;   o = al256(o + (size_t)(nc + 1) * 4);
         tab_bytes = o;
-        if (cudaMallocHost((void**)&tab_h, tab_bytes) != cudaSuccess) { tab_h = nullptr; return MANTRA_E_NOMEM; }
-        if (cudaMalloc((void**)&tab_d, tab_bytes) != cudaSuccess) { tab_d = nullptr; return MANTRA_E_NOMEM; }
-        if (cudaMallocHost((void**)&slot_h, (size_t)nc * SLOT_BYTES) != cudaSuccess) { slot_h = nullptr; return MANTRA_E_NOMEM; }
-        if (cudaMalloc((void**)&slot_d, (size_t)nc * SLOT_BYTES) != cudaSuccess) { slot_d = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<PinnedMemory>((void**)&tab_h, tab_bytes)) return MANTRA_E_NOMEM;
+        if (!take_memory<CudaMemory>((void**)&tab_d, tab_bytes)) return MANTRA_E_NOMEM;
+        if (!take_memory<PinnedMemory>((void**)&slot_h, (size_t)nc * SLOT_BYTES)) return MANTRA_E_NOMEM;
+        if (!take_memory<CudaMemory>((void**)&slot_d, (size_t)nc * SLOT_BYTES)) return MANTRA_E_NOMEM;
         std::memset(tab_h, 0, tab_bytes);
         cap = nc;
         invalidate_graph();
@@ -487,7 +465,7 @@ struct Engine {
         const size_t region = hop_region_bytes(n, A, &hws);
         const size_t budget = (size_t)((double)free_device_bytes() * 0.45);
         if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (cudaMalloc(&hop_mem, (size_t)grid * region) != cudaSuccess) { hop_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&hop_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(hop_mem, 0, (size_t)grid * region, sa));
         hws.base = hop_mem;
         hws.stride = region;
@@ -555,7 +533,7 @@ struct Engine {
         // MANTRA_BFS_GRID caps the resident CTAs
         if (const char* env = std::getenv("MANTRA_BFS_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
         if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (cudaMalloc(&bfs_mem, (size_t)grid * region) != cudaSuccess) { bfs_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&bfs_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(bfs_mem, 0, (size_t)grid * region, sa));
         bws.base = bfs_mem;
         bws.stride = region;
@@ -588,7 +566,7 @@ struct Engine {
         const size_t budget = free_device_bytes() / 3;
         uint64_t w = std::min<uint64_t>(warps, std::max<size_t>(budget / region, (size_t)wpb));
         const int blocks = (int)((w + wpb - 1) / wpb);
-        if (cudaMalloc(&pfm_mem, (size_t)blocks * wpb * region) != cudaSuccess) { pfm_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&pfm_mem, (size_t)blocks * wpb * region)) return MANTRA_E_NOMEM;
         pws.base = pfm_mem;
         pws.stride = region;
         pfm_grid = blocks;
@@ -629,7 +607,7 @@ struct Engine {
         if (const char* env = std::getenv("MANTRA_PFM_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
         const size_t budget = free_device_bytes() / 3;
         if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (cudaMalloc(&pc_mem, (size_t)grid * region) != cudaSuccess) { pc_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&pc_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         pcws.base = pc_mem;
         pcws.stride = region;
         for (int s = 0; s < 2; ++s)
@@ -653,7 +631,7 @@ struct Engine {
         const size_t region = sweep_region_bytes(n, m, &sws);
         const size_t budget = std::min<size_t>((size_t)16 << 30, free_device_bytes() / 10);
         const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 32, budget / region));
-        if (cudaMalloc(&sw_mem, (size_t)grid * region) != cudaSuccess) { sw_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&sw_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         sws.base = sw_mem;
         sws.stride = region;
         sw_regions = grid;
@@ -670,7 +648,7 @@ struct Engine {
         uint64_t cap = std::max<uint64_t>(sw_order_cap, 1u << 16);
         while (cap < units * 32) cap *= 2;
         if (sw_order) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_order); sw_order = nullptr; sw_order_cap = 0; }
-        if (cudaMalloc((void**)&sw_order, cap * 4) != cudaSuccess) { sw_order = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&sw_order, cap * 4)) return MANTRA_E_NOMEM;
         sw_order_cap = cap;
         invalidate_graph();
         return MANTRA_OK;
@@ -701,7 +679,7 @@ struct Engine {
         CU(scan_configure(smem_optin));
         const size_t region = scan_region_bytes(n, &scws);
         const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 2, free_device_bytes() / 6 / region));
-        if (cudaMalloc(&sc_mem, (size_t)grid * region) != cudaSuccess) { sc_mem = nullptr; return MANTRA_E_NOMEM; }
+        if (!take_memory<CudaMemory>((void**)&sc_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(sc_mem, 0, (size_t)grid * region, sa));
         scws.base = sc_mem;
         scws.stride = region;
@@ -1001,7 +979,6 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     if (rc == MANTRA_OK && any_s) rc = E.ensure_sweep_order(sunits);
     if (rc == MANTRA_OK && any_n) rc = E.ensure_scan(nn);
     if (rc == MANTRA_E_NOMEM) {
-        (void)cudaGetLastError();
         E.search_only = true;
         rc = run_tick(E, items, wide, out);
         E.search_only = false;
