@@ -172,7 +172,9 @@ bool few_choices(const mantra_graph* G) { return (uint64_t)G->A * 100 >= (uint64
 // under 2^16 edges: k_pfm_cta takes 0.1 us a sample there, and the cut would be
 // a tenth of the load.  Nor graphs in which ways back have
 // choices (few_choices).  MANTRA_PFM_KERNEL=sweep at the load lifts the last three.
-// Nor streams of more waves than a 32-bit place can name (waves_indexable).
+// Nor streams of more waves than a 32-bit place can name (waves_indexable), or
+// whose waves (up to 256 B an edge) find no room or would take more than a
+// quarter of what is free: the search needs none, and later calls need the rest.
 int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
@@ -180,7 +182,7 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
     if (m < (force ? 1u : 1u << 16) || !(force || few_choices(G)) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
     const size_t bytes = wave_tmp_bytes(m, G->A);
     char* tmp = (char*)pool.get(bytes);
-    if (!tmp) return MANTRA_E_NOMEM;
+    if (!tmp) return MANTRA_OK;
     uint32_t head[2] = {0, 1};
     int rc = MANTRA_OK;
     if (launch_wave_cut(G->dg, tmp, st) != cudaSuccess ||
@@ -189,13 +191,10 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
         rc = MANTRA_E_CUDA;
     if (rc == MANTRA_OK && head[1] == 0 && waves_indexable(head[0]) && (force || (uint64_t)head[0] * 2 <= (uint64_t)m)) {
         G->b_wmem = wave_bytes(head[0]);
-        G->wmem = pool.get(G->b_wmem);
-        if (!G->wmem) {
-            rc = MANTRA_E_NOMEM;
-        } else if (launch_wave_fill(&G->dg, tmp, head[0], (char*)G->wmem, st) != cudaSuccess ||
-                   cudaStreamSynchronize(st) != cudaSuccess) {
+        if (G->b_wmem <= (size_t)64 << 20 || G->b_wmem <= free_device_bytes() / 4) G->wmem = pool.get(G->b_wmem);
+        if (G->wmem && (launch_wave_fill(&G->dg, tmp, head[0], (char*)G->wmem, st) != cudaSuccess ||
+                        cudaStreamSynchronize(st) != cudaSuccess))
             rc = MANTRA_E_CUDA;
-        }
     }
     pool.put(tmp, bytes);
     return rc;
@@ -203,7 +202,8 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
 
 // The stream's chunks for k_scan, where its shared-memory bits can hold the
 // graph, no time step exceeds a chunk, and few edges share an arrival slot
-// (MANTRA_PFM_KERNEL=scan at the load lifts the last).
+// (MANTRA_PFM_KERNEL=scan at the load lifts the last).  Without room for them
+// the graph has none: the search needs none.
 int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
@@ -214,7 +214,7 @@ int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t
     const size_t nc = ((size_t)m + SCAN_CHUNK - 1) / SCAN_CHUNK;
     G->b_smem = al256((size_t)m * 4) + al256((nc + 1) * 4) + 256;
     G->smem = pool.get(G->b_smem);
-    if (!G->smem) return MANTRA_E_NOMEM;
+    if (!G->smem) return MANTRA_OK;
     uint32_t* slot = (uint32_t*)G->smem;
     uint32_t* ptr = (uint32_t*)((char*)G->smem + al256((size_t)m * 4));
     uint32_t* big = (uint32_t*)((char*)ptr + al256((nc + 1) * 4));
@@ -227,6 +227,9 @@ int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t
         G->dg.st_slot = slot;
         G->dg.scan_ptr = ptr;
         G->dg.n_scan = (uint32_t)nc;
+    } else {
+        pool.put(G->smem, G->b_smem);
+        G->smem = nullptr;
     }
     return MANTRA_OK;
 }

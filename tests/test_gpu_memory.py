@@ -1,0 +1,66 @@
+"""Calls on a device that other allocations have nearly filled, and what the
+library holds after a graph is freed: what a call can do without, it does
+without, and the results stay the same."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def M():
+    from paper_2304_08356_gb300 import build as B
+    B.build()
+    from paper_2304_08356_gb300 import mantra
+    return mantra
+
+
+def free_bytes():
+    import torch
+    return torch.cuda.mem_get_info()[0]
+
+
+class Filler:
+    """Leaves about `left` bytes of the device free."""
+
+    def __init__(self, left):
+        import torch
+        torch.cuda.empty_cache()
+        self.x = torch.empty(max(free_bytes() - left, 1 << 20), dtype=torch.uint8, device="cuda")
+
+    def release(self):
+        import torch
+        self.x = None
+        torch.cuda.empty_cache()
+
+
+def few_heads(n=200, m=2000000, heads=8, seed=1):
+    """Contacts at distinct times into a few heads: waves of about four edges, so
+    that the waves take more memory than the graph."""
+    rng = np.random.default_rng(seed)
+    v = rng.integers(0, heads, m)
+    u = (v + 1 + rng.integers(0, n - 1, m)) % n
+    return tuple(x.astype(np.uint32) for x in (u, v, np.arange(m) + 1))
+
+
+def test_load_without_room_for_waves(M, monkeypatch):
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    tri = few_heads()
+    M.Graph(*few_heads(m=70000), n=200).free()          # the library's own start
+    before = free_bytes()
+    g = M.Graph(*tri, n=200)
+    size = before - free_bytes()
+    fill = Filler(int(size * 0.6))                      # room for the store, not for its waves
+    try:
+        h = M.Graph(*tri, n=200)
+    finally:
+        fill.release()
+    _, want, info = g.estimate(2, 0.05, 0.1, 3, fixed_r=300)
+    assert info["edges_expanded"] == 0                  # swept
+    _, got, info = h.estimate(2, 0.05, 0.1, 3, fixed_r=300)
+    assert info["edges_expanded"] > 0                   # searched: it has no waves
+    assert want.sum() > 0 and np.array_equal(got, want)
+    for opt in (0, 1):
+        assert np.array_equal(h.estimate(opt, 0.05, 0.1, 3, fixed_r=300)[1], g.estimate(opt, 0.05, 0.1, 3, fixed_r=300)[1])
+    g.free()
+    h.free()
