@@ -307,12 +307,13 @@ struct Engine {
     std::map<uint64_t, int> hop_occ;       // (shape, shared nodes) -> CTAs per SM
     int tick_hop_nt = 256, tick_hop_sm = 0, tick_hop_cls = 0;
     uint32_t tick_hop_n = 0;
-    // pfm sweeps (k_sweep): a region per resident CTA (one warp, 32 samples);
-    // shared memory sized by the tick's graphs
-    char* sw_mem = nullptr; SweepWs sws{}; uint32_t sw_n = 0, sw_m = 0;
-    int sw_regions = 0, tick_sw_cls = 0;
+    // pfm sweeps (k_sweep): one allocation, laid out for the graphs of the tick as a
+    // region per resident CTA (one warp, 32 samples); shared memory and regions
+    // are sized by steps of their node and edge counts
+    char* sw_mem = nullptr; size_t sw_bytes = 0;
+    struct SweepPlan { uint32_t n = 0; int n_cls = 0, m_cls = 0, ctas = 0; size_t bytes = 0; SweepWs ws{}; };
+    SweepPlan tick_sw;                     // bytes: the allocation it wants (0: the present one)
     uint32_t* sw_order = nullptr; uint64_t sw_order_cap = 0; bool tick_sw_order = false;
-    uint32_t tick_sw_n = 0;
     std::map<uint32_t, int> sw_occ;        // shared nodes -> CTAs per SM
     bool tick_s = false;
     // pfm scans (k_scan): a region per resident CTA
@@ -379,24 +380,25 @@ struct Engine {
         if (tick_b) key |= (shape_of(tick_bfs_nt) << 3) | (tick_bfs_sm << 5);
         if (tick_h) key |= (shape_of(tick_hop_nt) << 6) | (tick_hop_sm << 8) | ((tick_hop_sm ? tick_hop_cls : 0) << 13);
         if (tick_p) key |= ((tick_cta ? 1 : 0) << 9) | ((tick_pc_nt == 256 ? 0 : 1) << 10) | (tick_pc_sm << 11);
-        if (tick_s) key |= (1 << 21) | (tick_sw_cls << 22) | ((tick_sw_order ? 1 : 0) << 30);
+        if (tick_s) key |= (1 << 21) | (tick_sw.n_cls << 22) | ((tick_sw_order ? 1 : 0) << 30) | ((uint64_t)tick_sw.m_cls << 41);
         if (tick_n) key |= (1ull << 31) | ((uint64_t)tick_sc_cls << 32) | ((uint64_t)(tick_sc_nt == 1024) << 40);
         return key;
     }
 
-    // A node count rounded up by at most an eighth, and the number of its step:
-    // shared-memory state is sized in these steps, so that a tick's launch
-    // configurations (captured graphs) stay few.
-    static uint32_t node_step(uint32_t n, int* cls) {
-        uint32_t nq = 64;
+    // A count rounded up by at most an eighth, and the number of its step (below
+    // 255): shared-memory state and k_sweep's regions are sized in these steps, so
+    // that a tick's launch configurations (captured graphs) stay few.
+    static uint64_t count_step(uint32_t n, int* cls) {
+        uint64_t nq = 64;
         int c = 0;
-        for (uint32_t step = 8; nq < n && c < 255; ++c) {
+        for (uint64_t step = 8; nq < n && c < 255; ++c) {
             nq += step;
             if (nq >= 16 * step) step *= 2;
         }
         *cls = c;
         return nq;
     }
+    static uint32_t node_step(uint32_t n, int* cls) { return (uint32_t)std::min<uint64_t>(count_step(n, cls), NONE); }
 
     // Table block layout: header | work counters | unit starts and tasks (bfs, pfm,
     // hop, sweep, scan) | reduction items | reduction row starts.
@@ -623,23 +625,49 @@ struct Engine {
         return MANTRA_OK;
     }
 
-    // pfm sweeps: one region per resident CTA of a small graph, at most 16 GB or a
-    // tenth of free memory.
-    int ensure_sweep(uint32_t n, uint32_t m) {
-        if (sw_mem && n <= sw_n && m <= sw_m) return MANTRA_OK;
-        n = std::max(n, sw_n);
-        m = std::max(m, sw_m);
-        if (sw_mem) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_mem); sw_mem = nullptr; }
-        CU(sweep_configure(smem_optin - sweep_static_smem()));
-        const size_t region = sweep_region_bytes(n, m, &sws);
-        const size_t budget = std::min<size_t>((size_t)16 << 30, free_device_bytes() / 10);
-        const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 32, budget / region));
-        if (!take_memory<CudaMemory>((void**)&sw_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
-        sws.base = sw_mem;
-        sws.stride = region;
-        sw_regions = grid;
-        sw_n = n; sw_m = m;
-        invalidate_graph();
+    // pfm sweeps of graphs of at most n nodes and m edges: the layout of a region, the
+    // CTAs that run (of those that the SMs hold, as many as there are regions for)
+    // and, where too few fit in the present allocation, the one to make: at most
+    // 16 GB or a tenth of free memory.
+    SweepPlan sweep_plan(uint32_t n, uint32_t m) {
+        SweepPlan p;
+        p.n = node_step(n, &p.n_cls);
+        if (!sweep_per_sm(p.n)) {                            // near the limit: the largest count that fits
+            uint32_t lo = 0, hi = p.n;
+            while (hi - lo > 1) {
+                const uint32_t mid = lo + (hi - lo) / 2;
+                if (sweep_smem_bytes(mid) + sweep_static_smem() <= smem_optin) lo = mid; else hi = mid;
+            }
+            p.n = std::max(lo, n);
+            p.n_cls = 255;
+        }
+        const size_t region = sweep_region_bytes(p.n, count_step(m, &p.m_cls), &p.ws);
+        const size_t want = (size_t)std::max(1, sweep_per_sm(p.n) * num_sms);
+        size_t have = sw_mem ? sw_bytes / region : 0;
+        if (have < want) {
+            // a new allocation for all CTAs, or for a quarter more than now (256 MB at
+            // least, so that growing graphs do not allocate every time)
+            const size_t budget = std::min<size_t>((size_t)16 << 30, (free_device_bytes() + sw_bytes) / 10);
+            const size_t bytes = std::max(region, std::min(std::max<size_t>(want * region, (size_t)256 << 20), budget));
+            if (have == 0 || bytes / region >= want || bytes / 5 * 4 >= sw_bytes) { p.bytes = bytes; have = bytes / region; }
+        }
+        p.ctas = (int)std::min(have, want);
+        p.ws.stride = region;
+        p.ws.n_smem = p.n;
+        return p;
+    }
+
+    int ensure_sweep(const SweepPlan& p) {
+        if (p.bytes) {
+            if (sw_mem) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_mem); sw_mem = nullptr; }
+            sw_bytes = 0;
+            CU(sweep_configure(smem_optin - sweep_static_smem()));
+            if (!take_memory<CudaMemory>((void**)&sw_mem, p.bytes)) return MANTRA_E_NOMEM;
+            sw_bytes = p.bytes;
+            invalidate_graph();
+        }
+        tick_sw = p;
+        tick_sw.ws.base = sw_mem;
         return MANTRA_OK;
     }
 
@@ -671,8 +699,6 @@ struct Engine {
         }
         return it->second;
     }
-
-    int sweep_grid(uint32_t nsm) { return std::min(sw_regions, sweep_per_sm(nsm) * num_sms); }
 
     // pfm scans: one region per CTA of the largest grid (two per SM).
     int ensure_scan(uint32_t n) {
@@ -735,11 +761,10 @@ struct Engine {
         if (tick_b || tick_h) CU(cudaEventRecord(e_b1, sa));
         if (tick_p || tick_s || tick_n) CU(cudaEventRecord(e_p0, sb));
         if (tick_s) {
-            SweepWs w = sws;
-            w.n_smem = tick_sw_n;
+            SweepWs w = tick_sw.ws;
             w.order = tick_sw_order ? sw_order : nullptr;
             CU(launch_sweep((const Task*)(tab_d + o_ts), (const uint64_t*)(tab_d + o_us), hdr + 4, work + 3, w,
-                            sweep_grid(tick_sw_n), sb));
+                            tick_sw.ctas, sb));
         }
         if (tick_n) {
             ScanWs w = scws;
@@ -900,31 +925,32 @@ bool can_sweep(const TickItem& it) {
 
 // Whether a tick's pfm samples take the sweep where they can.  The sweep's time
 // is that of the longest stream (one warp, 75 ns a wave), or its warps' waves
-// spread over the resident CTAs (ordered samples skip part of them, about what a
+// spread over the CTAs that run, for which its workspace has regions (ordered samples skip part of them, about what a
 // full GPU adds); the CTA kernel's, a graph-sized latency and a share per sample.
 // Measured (ms, sweep / CTA): n = 20,000 bursty 231 samples 2.7 / 0.79, 42,000
 // samples 9.1 / 33.4; n = 5,000 231: 1.1 / 0.22, 10,000: 1.39 / 2.53; n = 1,000
 // 2,000: 0.54 / 0.37; n = 50,000 uniform 231: 5.4 / 2.0, 8,000: 12.3 / 41.0.
 // MANTRA_PFM_KERNEL=sweep|cta|lane forces one of them.
-bool use_sweep(Engine& E, const std::vector<TickItem>& items) {
-    uint32_t n = 0;
+bool use_sweep(Engine& E, const std::vector<TickItem>& items, Engine::SweepPlan* plan) {
+    uint32_t n = 0, m_max = 0;
     double longest = 0, waves = 0, base = 0, samples = 0;
     for (const TickItem& it : items) {
         if (!can_sweep(it)) continue;
         const double w = 75e-6 * it.G->dg.n_waves, m = it.G->m, r = (double)it.job.count;
         n = std::max(n, it.G->n);
+        m_max = std::max(m_max, it.G->m);
         longest = std::max(longest, w);
         waves += w * std::ceil(r / 32.0);
         base = std::max(base, 0.08 + 1.2e-6 * m);
         samples += r * (8e-5 + 1.4e-9 * m);
     }
     if (!n) return false;
-    if (const char* env = std::getenv("MANTRA_PFM_KERNEL")) {
-        return std::strcmp(env, "sweep") == 0;
-    }
-    int cls = 0;
-    const int per = std::max(1, E.sweep_per_sm(Engine::node_step(n, &cls)));
-    return 0.2 + std::max(1.3 * longest, waves / ((double)per * E.num_sms)) < base + samples;
+    const char* env = std::getenv("MANTRA_PFM_KERNEL");
+    if (env && std::strcmp(env, "sweep") != 0) return false;
+    // even on every SM it would take longer: its workspace is not looked at
+    if (!env && 0.2 + 1.3 * longest >= base + samples) return false;
+    *plan = E.sweep_plan(n, m_max);
+    return env || 0.2 + std::max(1.3 * longest, waves / (double)plan->ctas) < base + samples;
 }
 
 // One tick over `items` (narrow kernels, captured graph), or with `wide` the
@@ -941,17 +967,17 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     uint64_t hsamples = 0;
     const mantra_graph* gh = nullptr;   // the tick's largest k_hop graph
     bool any_s = false;
-    uint32_t sn = 0, smx = 0;
     uint64_t sunits = 0, nsamples = 0;
     bool any_n = false;
     uint32_t nn = 0;
     std::vector<char> sweep(k, 0);
-    const bool sweeps = !wide && !E.search_only && use_sweep(E, items);
+    Engine::SweepPlan plan;
+    const bool sweeps = !wide && !E.search_only && use_sweep(E, items, &plan);
     for (uint32_t x = 0; x < k; ++x) {
         const TickItem& it = items[x];
         if (sweeps && can_sweep(it)) {
             sweep[x] = 1;
-            any_s = true; sn = std::max(sn, it.G->n); smx = std::max(smx, it.G->m);
+            any_s = true;
             sunits += (it.job.count + 31) / 32;
         } else if (!wide && !E.search_only && use_scan(E, it)) {
             sweep[x] = 2;
@@ -978,7 +1004,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
     // a device too full for the workspaces of the passes over the stream runs the
     // search, whose workspace may be there already
-    rc = any_s ? E.ensure_sweep(sn, smx) : MANTRA_OK;
+    rc = any_s ? E.ensure_sweep(plan) : MANTRA_OK;
     if (rc == MANTRA_OK && any_s) rc = E.ensure_sweep_order(sunits);
     if (rc == MANTRA_OK && any_n) rc = E.ensure_scan(nn);
     if (rc == MANTRA_E_NOMEM) {
@@ -988,15 +1014,6 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         return rc;
     }
     if (rc != MANTRA_OK) return rc;
-    if (any_s) {
-        E.tick_sw_n = Engine::node_step(sn, &E.tick_sw_cls);
-        // near the limit the step may not fit: the graphs' own size then (a graph with
-        // waves fits), captured as the last step
-        if (!E.sweep_grid(E.tick_sw_n)) {
-            E.tick_sw_n = E.sw_n;
-            E.tick_sw_cls = 255;
-        }
-    }
     if (any_n) {
         E.tick_sc_n = Engine::node_step(nn, &E.tick_sc_cls);
         // CTA size, ms with 512 and 1,024 threads: few samples want each of them fast

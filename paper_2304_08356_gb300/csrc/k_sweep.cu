@@ -592,7 +592,7 @@ __global__ void __launch_bounds__(1024) k_sweep_order(const Task* tasks, const u
 
 // Region of one CTA: the log holds a record per edge at most (edges of one slot
 // may bring the same samples).
-size_t sweep_region_bytes(uint32_t n, uint32_t m, SweepWs* ws) {
+size_t sweep_region_bytes(uint32_t n, uint64_t m, SweepWs* ws) {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     ws->path_cap = std::min<uint32_t>(n + 2, 2048);
     ws->cone_cap = std::min<uint32_t>(n + 1, 1024);

@@ -873,7 +873,7 @@ cudaError_t launch_scan(const Task* tasks, const uint64_t* unit_start, const uin
                         const ScanWs& ws, int grid, cudaStream_t st);
 // Fills st_slot (m), scan_ptr (ceil(m / SCAN_CHUNK) + 1) and *big (a chunk would exceed 2,048 edges: no scan).
 cudaError_t launch_scan_maps(const DevGraph& g, uint32_t* st_slot, uint32_t* ptr, uint32_t* big, cudaStream_t st);
-size_t sweep_region_bytes(uint32_t n, uint32_t m, SweepWs* ws);
+size_t sweep_region_bytes(uint32_t n, uint64_t m, SweepWs* ws);
 size_t sweep_smem_bytes(uint32_t n);
 size_t sweep_static_smem();
 cudaError_t sweep_configure(size_t smem);

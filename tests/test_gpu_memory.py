@@ -64,3 +64,28 @@ def test_load_without_room_for_waves(M, monkeypatch):
         assert np.array_equal(h.estimate(opt, 0.05, 0.1, 3, fixed_r=300)[1], g.estimate(opt, 0.05, 0.1, 3, fixed_r=300)[1])
     g.free()
     h.free()
+
+
+def test_sweep_after_a_dense_graph(M, monkeypatch):
+    """One pfm call on a graph of many edges, whose sweep takes 160 MB a warp, does
+    not slow the calls on other graphs down (with a workspace that kept that
+    layout they had a tenth of the warps)."""
+    from paper_2304_08356_gb300 import synth
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    g = M.Graph(*synth.chung_lu_bursty(n=5000, m=125000, seed=3))
+
+    def run():
+        res = [g.estimate(2, 0.05, 0.1, 3, fixed_r=60000)[1:] for _ in range(5)]
+        assert all(i["edges_expanded"] == 0 for _, i in res)
+        return res[0][0], min(i["kernel_ms"] for _, i in res)
+    hits, ms = run()
+    rng = np.random.default_rng(5)
+    n, m = 50000, 10000000
+    u = rng.integers(0, n, m)
+    dense = M.Graph(u.astype(np.uint32), ((u + 1 + rng.integers(0, n - 1, m)) % n).astype(np.uint32),
+                    np.arange(1, m + 1).astype(np.uint32), n=n)
+    assert dense.estimate(2, 0.05, 0.1, 3, fixed_r=64)[2]["edges_expanded"] == 0
+    again, ms2 = run()
+    assert np.array_equal(hits, again) and ms2 < 2 * ms
+    dense.free()
+    g.free()
