@@ -329,7 +329,11 @@ int mantra_sample_paths_noalloc(const mantra_graph* g, mantra_opt opt, uint64_t 
  * (sh/sfm) or six (pfm) CTAs per SM (per CTA about 28 bytes per arrival
  * slot and 28 per node for sh/sfm, at least 10 and 70 with small graphs' path
  * sets; with RTB or fsfm requests also 44 and 52; 56 per node plus 4 per unit
- * of the graph's path-count bound for pfm), and fewer than `max_active` (0 = 256) run; a request is always admitted when none is
+ * of the graph's path-count bound for pfm); pfm requests on graphs that the
+ * passes over the time-sorted edges can take add 16 bytes per edge for every
+ * warp that the SMs' shared memory holds (64 MB more, at most 16 GB) and 72 per
+ * node for every SM.  Fewer than `max_active` (0 = 256) run; a request is
+ * always admitted when none is
  * running.  Each tick launches the pending samples of every running request
  * together; finished requests leave between ticks and queued ones join at the
  * next tick.  A request's result equals mantra_estimate on the same

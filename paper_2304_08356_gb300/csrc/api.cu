@@ -436,22 +436,40 @@ struct Engine {
         return MANTRA_OK;
     }
 
-    // Device bytes of the search workspaces for graphs with these maxima (sh/sfm:
-    // n, A, slots per vertex; with full also k_bfs, which RTB and fsfm run on,
-    // and its RTB scratch; pfm: n, cbound), at the largest grid of any CTA shape
-    // (256-thread CTAs: four per SM for k_hop and k_bfs, six for k_pfm_cta) and
-    // without the free-memory caps of ensure_hop / ensure_bfs / ensure_pfm_cta:
-    // an upper estimate of what those allocate.
-    size_t ws_estimate(uint32_t n, uint32_t A, uint32_t zc, bool full, uint32_t pn, uint32_t cb) const {
+    // The largest graphs of each search kernel among some requests: sh/sfm (with
+    // full also on k_bfs, which RTB and fsfm run on, and its RTB scratch), pfm,
+    // and the pfm graphs that k_sweep and k_scan can take.
+    struct WsGraphs {
+        uint32_t n = 0, A = 0, vslots = 0;
+        bool full = false;
+        uint32_t pfm_n = 0, pfm_cb = 0, sweep_n = 0, sweep_m = 0, scan_n = 0;
+    };
+
+    // Device bytes of the search workspaces for such graphs, at the largest grid of
+    // any CTA shape (256-thread CTAs: four per SM for k_hop and k_bfs, six for
+    // k_pfm_cta; k_sweep: what its shared memory admits, at most 16 GB; k_scan: two)
+    // and without the free-memory caps of the ensure_* functions: an upper estimate of
+    // what those allocate.  Reads nothing that a tick changes.
+    size_t ws_estimate(const WsGraphs& w) const {
         size_t b = 0;
         const size_t sms = (size_t)std::max(num_sms, 1);
-        if (n) {
+        if (w.n) {
             HopWs h{};
-            BfsWs w{};
-            const size_t hop = hop_region_bytes(n, A, &h), bfs = bfs_region_bytes(n, A, zc, false, full, &w);
-            b += 4 * sms * (full ? hop + bfs : std::max(hop, bfs));
+            BfsWs f{};
+            const size_t hop = hop_region_bytes(w.n, w.A, &h), bfs = bfs_region_bytes(w.n, w.A, w.vslots, false, w.full, &f);
+            b += 4 * sms * (w.full ? hop + bfs : std::max(hop, bfs));
         }
-        if (pn) { PfmCtaWs w{}; b += 6 * sms * pfm_cta_region_bytes(pn, cb, false, &w); }
+        if (w.pfm_n) { PfmCtaWs p{}; b += 6 * sms * pfm_cta_region_bytes(w.pfm_n, w.pfm_cb, false, &p); }
+        if (w.sweep_n) {
+            SweepWs p{};
+            int c = 0;
+            const size_t region = sweep_region_bytes(node_step(w.sweep_n, &c), count_step(w.sweep_m, &c), &p);
+            const size_t per = (smem_optin + 1024) / (sweep_smem_bytes(w.sweep_n) + sweep_static_smem() + 1024);
+            b += std::max(region, std::min<size_t>((size_t)16 << 30, std::max<size_t>((size_t)256 << 20,
+                                                   std::max<size_t>(1, std::min<size_t>(per, 32)) * sms * region)));
+            b += (size_t)64 << 20;                           // ordered samples (ensure_sweep_order)
+        }
+        if (w.scan_n) { ScanWs p{}; b += 2 * sms * scan_region_bytes(w.scan_n, &p); }
         return b;
     }
 
@@ -1644,21 +1662,23 @@ struct Server {
 
     // Search workspace for the running requests and (if given) one more.
     size_t ws_for(const Request* extra) const {
-        uint32_t n = 0, A = 0, z = 0, pn = 0, cb = 0;
-        bool dl = false;
+        Engine::WsGraphs w;
         auto add = [&](const Request* r) {
             const mantra_graph* G = r->p.G;
             if (!G) return;
             if (r->p.opt == MANTRA_PFM) {
-                pn = std::max(pn, G->n); cb = std::max(cb, G->dg.cbound);
+                w.pfm_n = std::max(w.pfm_n, G->n); w.pfm_cb = std::max(w.pfm_cb, G->dg.cbound);
+                if (r->p.estimator != 0) return;
+                if (G->dg.n_waves) { w.sweep_n = std::max(w.sweep_n, G->n); w.sweep_m = std::max(w.sweep_m, G->m); }
+                if (G->dg.n_scan) w.scan_n = std::max(w.scan_n, G->n);
             } else {
-                n = std::max(n, G->n); A = std::max(A, G->A); z = std::max(z, G->dg.max_vslots);
-                dl = dl || r->p.estimator == 2 || r->p.opt == MANTRA_FSFM;
+                w.n = std::max(w.n, G->n); w.A = std::max(w.A, G->A); w.vslots = std::max(w.vslots, G->dg.max_vslots);
+                w.full = w.full || r->p.estimator == 2 || r->p.opt == MANTRA_FSFM;
             }
         };
         for (const Request* r : active) add(r);
         if (extra) add(extra);
-        return E->ws_estimate(n, A, z, dl, pn, cb);
+        return E->ws_estimate(w);
     }
 
     void loop() {

@@ -89,3 +89,38 @@ def test_sweep_after_a_dense_graph(M, monkeypatch):
     assert np.array_equal(hits, again) and ms2 < 2 * ms
     dense.free()
     g.free()
+
+
+SERVE = """
+import numpy as np, torch
+from paper_2304_08356_gb300 import mantra as M, synth
+gs = [M.Graph(*synth.chung_lu_bursty(n=5000, m=125000, seed=3)), M.Graph(*synth.chung_lu_bursty(n=1000, m=20000, seed=4))]
+before = torch.cuda.mem_get_info()[0]
+srv = M.Server(hbm_budget=1 << 40)
+ids = [srv.submit(g, 2, eps, 0.1, 5) for g in gs for eps in (0.008, 0.01, 0.05)]
+seen, done = 0, 0
+while done < len(ids):
+    st = srv.stats()
+    if st["active"]:
+        seen = max(seen, st["bytes_in_use"])
+    done = st["finished"]
+for i in ids:
+    srv.wait(i, timeout=300)
+print("counted %d held %d" % (seen, before - torch.cuda.mem_get_info()[0]))
+srv.close()
+"""
+
+
+def test_admission_counts_what_is_allocated(M):
+    """In a fresh process: the device state that a server reports for its pfm
+    requests is no less than what serving them took."""
+    import os
+    import re
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", SERVE], capture_output=True, text=True, cwd=root)
+    assert r.returncode == 0, r.stderr
+    counted, held = map(int, re.search(r"counted (\d+) held (\d+)", r.stdout).groups())
+    assert held > 200 << 20                             # the sweep's workspace is part of it
+    assert counted >= held - (32 << 20)                 # (tables, captured launches)
