@@ -183,6 +183,11 @@ int mantra_graph_info(const mantra_graph* g, uint32_t* n, uint64_t* m_dedup, uin
 int mantra_graph_edges(const mantra_graph* g, uint32_t* u_out, uint32_t* v_out, uint32_t* t_out,
                        uint32_t* uedge_out, uint32_t* n_underlying);
 
+/* Frees g.  Its device memory goes back to the device, but for blocks that the next
+ * load may use (256 MB in all).  The search workspaces, sized for the largest
+ * graphs used and within shares of the free memory, and up to 8 GB of finished
+ * calls' buffers stay with the library; they make room for each other and for new
+ * graphs before a call answers MANTRA_E_NOMEM. */
 void mantra_graph_free(mantra_graph* g);
 
 /* Algorithm 1 (MANTRA): progressive sampling of (s,z) pairs with the

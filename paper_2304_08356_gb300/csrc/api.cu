@@ -91,7 +91,10 @@ struct PinnedMemory {
     static void clear() { (void)cudaGetLastError(); }
 };
 
-constexpr size_t kPoolCacheBytes = (size_t)8 << 30;
+// Blocks of finished problems and of freed graphs that stay cached: a load of a graph
+// of 500,000 edges is 3.5 ms, and a new block would be a tenth of that; a large
+// graph's memory goes back to the device when it is freed.
+constexpr size_t kPoolCacheBytes = (size_t)8 << 30, kGraphCacheBytes = (size_t)256 << 20;
 
 using DevPool = MemoryPool<CudaMemory>;
 
@@ -101,7 +104,12 @@ using DevPool = MemoryPool<CudaMemory>;
 // dense slot id).  The host team of store.cu builds the arrays; this uploads
 // them into one device allocation, each array from its page-locked buffer.
 // ---------------------------------------------------------------------------
-int upload_store(const StoreHost& H, mantra_graph* G, DevPool& pool, cudaStream_t st) {
+struct Engine;
+// A block of a graph, and back (Engine::block).  optional: the graph can do without.
+void* graph_block(Engine& E, size_t bytes, bool optional);
+void graph_unblock(Engine& E, void* p, size_t bytes);
+
+int upload_store(const StoreHost& H, mantra_graph* G, Engine& E, cudaStream_t st) {
     const uint32_t** dst[SA_COUNT] = {};
     dst[SA_OUT_PTR] = &G->dg.out_ptr;   dst[SA_OUT_V] = &G->dg.out_v;       dst[SA_OUT_T] = &G->dg.out_t;
     dst[SA_OUT_SLOT] = &G->dg.out_slot; dst[SA_SLOT_PTR] = &G->dg.slot_ptr; dst[SA_SLOT_T] = &G->dg.slot_t;
@@ -128,7 +136,7 @@ int upload_store(const StoreHost& H, mantra_graph* G, DevPool& pool, cudaStream_
     total += al256((size_t)nb * H.n * 8);
     const size_t o_dt = total;
     total += al256(32 * 4);
-    G->dmem = pool.get(total);
+    G->dmem = graph_block(E, total, false);
     if (!G->dmem) return MANTRA_E_NOMEM;
     G->b_dmem = total;
     size_t off = 0;
@@ -175,13 +183,13 @@ bool few_choices(const mantra_graph* G) { return (uint64_t)G->A * 100 >= (uint64
 // Nor streams of more waves than a 32-bit place can name (waves_indexable), or
 // whose waves (up to 256 B an edge) find no room or would take more than a
 // quarter of what is free: the search needs none, and later calls need the rest.
-int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
+int build_waves(mantra_graph* G, size_t smem_optin, Engine& E, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
     const bool force = env && std::strcmp(env, "sweep") == 0;
     if (m < (force ? 1u : 1u << 16) || !(force || few_choices(G)) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
     const size_t bytes = wave_tmp_bytes(m, G->A);
-    char* tmp = (char*)pool.get(bytes);
+    char* tmp = (char*)graph_block(E, bytes, true);
     if (!tmp) return MANTRA_OK;
     uint32_t head[2] = {0, 1};
     int rc = MANTRA_OK;
@@ -191,12 +199,13 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
         rc = MANTRA_E_CUDA;
     if (rc == MANTRA_OK && head[1] == 0 && waves_indexable(head[0]) && (force || (uint64_t)head[0] * 2 <= (uint64_t)m)) {
         G->b_wmem = wave_bytes(head[0]);
-        if (G->b_wmem <= (size_t)64 << 20 || G->b_wmem <= free_device_bytes() / 4) G->wmem = pool.get(G->b_wmem);
+        if (G->b_wmem <= (size_t)64 << 20 || G->b_wmem <= free_device_bytes() / 4)
+            G->wmem = graph_block(E, G->b_wmem, true);
         if (G->wmem && (launch_wave_fill(&G->dg, tmp, head[0], (char*)G->wmem, st) != cudaSuccess ||
                         cudaStreamSynchronize(st) != cudaSuccess))
             rc = MANTRA_E_CUDA;
     }
-    pool.put(tmp, bytes);
+    graph_unblock(E, tmp, bytes);
     return rc;
 }
 
@@ -204,7 +213,7 @@ int build_waves(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t 
 // graph, no time step exceeds a chunk, and few edges share an arrival slot
 // (MANTRA_PFM_KERNEL=scan at the load lifts the last).  Without room for them
 // the graph has none: the search needs none.
-int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t st) {
+int build_chunks(mantra_graph* G, size_t smem_optin, Engine& E, cudaStream_t st) {
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
     const bool force = env && std::strcmp(env, "scan") == 0;
@@ -213,7 +222,7 @@ int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t
         scan_smem_bytes(1024, G->n) > smem_optin) return MANTRA_OK;
     const size_t nc = ((size_t)m + SCAN_CHUNK - 1) / SCAN_CHUNK;
     G->b_smem = al256((size_t)m * 4) + al256((nc + 1) * 4) + 256;
-    G->smem = pool.get(G->b_smem);
+    G->smem = graph_block(E, G->b_smem, true);
     if (!G->smem) return MANTRA_OK;
     uint32_t* slot = (uint32_t*)G->smem;
     uint32_t* ptr = (uint32_t*)((char*)G->smem + al256((size_t)m * 4));
@@ -228,7 +237,7 @@ int build_chunks(mantra_graph* G, size_t smem_optin, DevPool& pool, cudaStream_t
         G->dg.scan_ptr = ptr;
         G->dg.n_scan = (uint32_t)nc;
     } else {
-        pool.put(G->smem, G->b_smem);
+        graph_unblock(E, G->smem, G->b_smem);
         G->smem = nullptr;
     }
     return MANTRA_OK;
@@ -303,7 +312,7 @@ struct Engine {
     // threads; the arrivals in shared memory are sized by the tick's graphs
     // (hop_nsm: their largest node count, rounded up)
     char* hop_mem = nullptr; HopWs hws{}; uint32_t hop_n = 0, hop_A = 0;
-    int hop_regions = 0;
+    int hop_regions = 0, hop_want = 0;     // regions allocated, and wanted then
     std::map<uint64_t, int> hop_occ;       // (shape, shared nodes) -> CTAs per SM
     int tick_hop_nt = 256, tick_hop_sm = 0, tick_hop_cls = 0;
     uint32_t tick_hop_n = 0;
@@ -342,7 +351,8 @@ struct Engine {
     // captured ticks, by launch configuration (tick_key)
     std::map<uint64_t, cudaGraphExec_t> gexec;
     bool use_graph = true;
-    DevPool pool{kPoolCacheBytes};
+    DevPool pool{kPoolCacheBytes}, graphs{kGraphCacheBytes};
+    bool in_tick = false;      // between the choice of a tick's kernels and the end of their work
 
     int init(int dev) {
         device = dev;
@@ -399,6 +409,56 @@ struct Engine {
         return nq;
     }
     static uint32_t node_step(uint32_t n, int* cls) { return (uint32_t)std::min<uint64_t>(count_step(n, cls), NONE); }
+
+    // Gives back the search workspaces that the tick in progress (if any) does not use;
+    // they are made again when a tick needs them.
+    void drop_idle() {
+        cudaStreamSynchronize(sb);
+        cudaStreamSynchronize(sa);
+        auto drop = [&](bool used, char** p) {
+            if (!*p || (in_tick && used)) return;
+            cudaFree(*p);
+            *p = nullptr;
+        };
+        drop(tick_h, &hop_mem);
+        drop(tick_b, &bfs_mem);
+        drop(tick_p && !tick_cta, &pfm_mem);
+        drop(tick_p && tick_cta, &pc_mem);
+        drop(tick_s, &sw_mem);
+        drop(tick_n, &sc_mem);
+        if (!hop_mem) { hop_n = hop_A = 0; hop_regions = hop_want = 0; }
+        if (!bfs_mem) { bfs_n = bfs_A = bfs_z = 0; bfs_dl = false; }
+        if (!pfm_mem) { pfm_n = pfm_lcap = 0; pfm_warps = 0; }
+        if (!pc_mem) { pc_n = pc_cb = 0; }
+        if (!sw_mem) sw_bytes = 0;
+        if (!sc_mem) sc_n = 0;
+        invalidate_graph();
+    }
+
+    // Device memory for a search workspace.  Before it fails, everything that only
+    // waits to be used again is given back: cached blocks, and other kernels'
+    // workspaces unless the caller can do without (optional).
+    bool alloc(char** p, size_t bytes, bool optional = false) {
+        if (take_memory<CudaMemory>((void**)p, bytes)) return true;
+        pool.release_all();
+        graphs.release_all();
+        if (take_memory<CudaMemory>((void**)p, bytes)) return true;
+        if (optional) return false;
+        drop_idle();
+        return take_memory<CudaMemory>((void**)p, bytes);
+    }
+
+    // A block of `from` (pool or graphs), with the same last resorts.
+    void* block(DevPool& from, size_t bytes, bool optional = false) {
+        void* p = from.get(bytes);
+        if (p) return p;
+        pool.release_all();
+        graphs.release_all();
+        p = from.get(bytes);
+        if (p || optional) return p;
+        drop_idle();
+        return from.get(bytes);
+    }
 
     // Table block layout: header | work counters | unit starts and tasks (bfs, pfm,
     // hop, sweep, scan) | reduction items | reduction row starts.
@@ -473,26 +533,42 @@ struct Engine {
         return b;
     }
 
-    // sh/sfm level search: one region per CTA of the largest resident grid, at
-    // most 45 % of free memory (k_bfs and the pfm kernels may need theirs beside it).
-    int ensure_hop(uint32_t n, uint32_t A) {
-        if (hop_mem && n <= hop_n && A <= hop_A) return MANTRA_OK;
+    // How many of `want` regions a search workspace gets: what `share` of the free
+    // memory holds, one at least.  With less than one per SM, memory that only waits
+    // to be used again is given back first.
+    int regions_for(int want, size_t region, double share) {
+        auto fit = [&]() { return (size_t)((double)free_device_bytes() * share) / region; };
+        size_t f = fit();
+        if (f < (size_t)std::min(want, num_sms)) {
+            pool.release_all();
+            graphs.release_all();
+            drop_idle();
+            f = fit();
+        }
+        return (int)std::max<size_t>(1, std::min<size_t>((size_t)want, f));
+    }
+
+    // sh/sfm level search: a region per CTA of the largest resident grid of any shape
+    // while that is at most 4 GB, else per CTA that the tick runs (n = 10^6 and m =
+    // 2*10^7: 152 CTAs and 41 GB, 160 GB for all shapes); at most 45 % of free memory
+    // (k_bfs and the pfm kernels may need theirs beside it).
+    int ensure_hop(uint32_t n, uint32_t A, int ctas) {
+        if (hop_mem && n <= hop_n && A <= hop_A && ctas <= hop_want) return MANTRA_OK;
         n = std::max(n, hop_n);
         A = std::max(A, hop_A);
+        int want = std::max(ctas, hop_want);
         if (hop_mem) { cudaStreamSynchronize(sa); cudaFree(hop_mem); hop_mem = nullptr; }
-        CU(hop_configure(smem_optin));
-        int grid = 1;
-        for (int nt : {256, 512, 1024}) grid = std::max(grid, hop_grid(nt, 0, INT_MAX));
-        // MANTRA_BFS_GRID caps the resident CTAs
-        if (const char* env = std::getenv("MANTRA_BFS_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
         const size_t region = hop_region_bytes(n, A, &hws);
-        const size_t budget = (size_t)((double)free_device_bytes() * 0.45);
-        if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (!take_memory<CudaMemory>((void**)&hop_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+        int all = 1;
+        for (int nt : {256, 512, 1024}) all = std::max(all, hop_grid(nt, 0, INT_MAX));
+        if ((size_t)all * region <= (size_t)4 << 30) want = all;
+        const int grid = regions_for(want, region, 0.45);
+        if (!alloc(&hop_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(hop_mem, 0, (size_t)grid * region, sa));
         hws.base = hop_mem;
         hws.stride = region;
         hop_regions = grid;
+        hop_want = want;
         hop_n = n; hop_A = A;
         invalidate_graph();
         return MANTRA_OK;
@@ -507,9 +583,12 @@ struct Engine {
         auto it = hop_occ.find(key);
         if (it == hop_occ.end()) {
             int per = 0;
-            if (hop_blocks_per_sm(nt, nsm > 0, smem, &per) != cudaSuccess) per = 0;
+            if (hop_configure(smem_optin) != cudaSuccess || hop_blocks_per_sm(nt, nsm > 0, smem, &per) != cudaSuccess)
+                per = 0;
             it = hop_occ.emplace(key, per).first;
         }
+        // MANTRA_BFS_GRID caps the resident CTAs
+        if (const char* env = std::getenv("MANTRA_BFS_GRID")) most = std::max(1, std::min(most, std::atoi(env)));
         return std::min(most, it->second * num_sms);
     }
 
@@ -548,15 +627,14 @@ struct Engine {
         // the search regions may take 60 % of free memory: on the n = 10^6,
         // m = 2*10^7 graph one region is about half a GB and every SM should
         // keep its resident CTAs
-        const size_t budget = (size_t)((double)free_device_bytes() * 0.6);
         int grid = 0;
         for (int s = 0; s < 3; ++s)
             for (int p = 0; p < 2; ++p) grid = std::max(grid, num_sms * per[s][p]);
         grid = std::max(grid, 1);
         // MANTRA_BFS_GRID caps the resident CTAs
         if (const char* env = std::getenv("MANTRA_BFS_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
-        if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (!take_memory<CudaMemory>((void**)&bfs_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+        grid = regions_for(grid, region, 0.6);
+        if (!alloc(&bfs_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(bfs_mem, 0, (size_t)grid * region, sa));
         bws.base = bfs_mem;
         bws.stride = region;
@@ -589,7 +667,7 @@ struct Engine {
         const size_t budget = free_device_bytes() / 3;
         uint64_t w = std::min<uint64_t>(warps, std::max<size_t>(budget / region, (size_t)wpb));
         const int blocks = (int)((w + wpb - 1) / wpb);
-        if (!take_memory<CudaMemory>((void**)&pfm_mem, (size_t)blocks * wpb * region)) return MANTRA_E_NOMEM;
+        if (!alloc(&pfm_mem, (size_t)blocks * wpb * region)) return MANTRA_E_NOMEM;
         pws.base = pfm_mem;
         pws.stride = region;
         pfm_grid = blocks;
@@ -628,9 +706,8 @@ struct Engine {
             for (int p = 0; p < 4; ++p) grid = std::max(grid, num_sms * per[s][p]);
         grid = std::max(grid, 1);
         if (const char* env = std::getenv("MANTRA_PFM_GRID")) grid = std::max(1, std::min(grid, std::atoi(env)));
-        const size_t budget = free_device_bytes() / 3;
-        if ((size_t)grid * region > budget) grid = (int)std::max<size_t>(1, budget / region);
-        if (!take_memory<CudaMemory>((void**)&pc_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+        grid = regions_for(grid, region, 1.0 / 3.0);
+        if (!alloc(&pc_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
         pcws.base = pc_mem;
         pcws.stride = region;
         for (int s = 0; s < 2; ++s)
@@ -680,7 +757,7 @@ struct Engine {
             if (sw_mem) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_mem); sw_mem = nullptr; }
             sw_bytes = 0;
             CU(sweep_configure(smem_optin - sweep_static_smem()));
-            if (!take_memory<CudaMemory>((void**)&sw_mem, p.bytes)) return MANTRA_E_NOMEM;
+            if (!alloc(&sw_mem, p.bytes, true)) return MANTRA_E_NOMEM;
             sw_bytes = p.bytes;
             invalidate_graph();
         }
@@ -697,7 +774,7 @@ struct Engine {
         uint64_t cap = std::max<uint64_t>(sw_order_cap, 1u << 16);
         while (cap < units * 32) cap *= 2;
         if (sw_order) { cudaStreamSynchronize(sb); cudaStreamSynchronize(sa); cudaFree(sw_order); sw_order = nullptr; sw_order_cap = 0; }
-        if (!take_memory<CudaMemory>((void**)&sw_order, cap * 4)) return MANTRA_E_NOMEM;
+        if (!alloc((char**)&sw_order, cap * 4, true)) return MANTRA_E_NOMEM;
         sw_order_cap = cap;
         invalidate_graph();
         return MANTRA_OK;
@@ -726,7 +803,7 @@ struct Engine {
         CU(scan_configure(smem_optin));
         const size_t region = scan_region_bytes(n, &scws);
         const int grid = (int)std::max<size_t>(1, std::min<size_t>((size_t)num_sms * 2, free_device_bytes() / 6 / region));
-        if (!take_memory<CudaMemory>((void**)&sc_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+        if (!alloc(&sc_mem, (size_t)grid * region, true)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(sc_mem, 0, (size_t)grid * region, sa));
         scws.base = sc_mem;
         scws.stride = region;
@@ -843,6 +920,9 @@ struct Engine {
 
 std::mutex g_engines_mu;
 Engine* g_engines[64];
+
+void* graph_block(Engine& E, size_t bytes, bool optional) { return E.block(E.graphs, bytes, optional); }
+void graph_unblock(Engine& E, void* p, size_t bytes) { E.graphs.put(p, bytes); }
 
 int engine_for(int dev, Engine** out) {
     if (dev < 0 || dev >= 64) return MANTRA_E_CUDA;
@@ -1019,7 +1099,12 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     }
     E.tick_b = any_b; E.tick_h = any_h; E.tick_p = any_p; E.tick_s = any_s; E.tick_n = any_n;
     const bool cta = any_p && !wide && pfm_use_cta();
-    if (any_h && (rc = E.ensure_hop(hn, hA)) != MANTRA_OK) return rc;
+    E.tick_cta = cta;
+    struct InTick {
+        bool& on;
+        explicit InTick(bool& b) : on(b) { on = true; }
+        ~InTick() { on = false; }
+    } in_tick(E.in_tick);
     // a device too full for the workspaces of the passes over the stream runs the
     // search, whose workspace may be there already
     rc = any_s ? E.ensure_sweep(plan) : MANTRA_OK;
@@ -1047,7 +1132,6 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     if (any_b && (rc = E.ensure_bfs(bn, bA, bz, dl)) != MANTRA_OK) return rc;
     if (any_p && cta && (rc = E.ensure_pfm_cta(pn, plc)) != MANTRA_OK) return rc;
     if (any_p && !cta && (rc = E.ensure_pfm(pn, plc, pwarps)) != MANTRA_OK) return rc;
-    E.tick_cta = cta;
     // k_hop: CTA shape and placement of the arrivals.  Measured (sh / sfm, ms for
     // 8,000 to 22,000 samples; threads:1 in shared memory, :0 in global memory):
     //   n = 5,000 bursty    256:1 0.85   512:1 1.20   256:0 1.13   1024:0 2.29
@@ -1064,7 +1148,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     if (any_h) {
         int cls = 0;
         const uint32_t nq = Engine::node_step(hn, &cls);
-        auto grid = [&](int nt, int sm) { return E.hop_grid(nt, sm ? nq : 0, E.hop_regions); };
+        auto grid = [&](int nt, int sm) { return E.hop_grid(nt, sm ? nq : 0, INT_MAX); };
         int nt = 1024, sm = 0;
         if (hsamples <= 2ull * (uint64_t)E.num_sms) {
             nt = hn > 12000 ? 1024 : (hn > 1500 ? 512 : 256);
@@ -1085,6 +1169,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         E.tick_hop_sm = sm;
         E.tick_hop_cls = cls;
         E.tick_hop_n = nq;
+        if ((rc = E.ensure_hop(hn, hA, grid(nt, sm))) != MANTRA_OK) return rc;
     }
     // k_bfs CTA shape: 1024 threads for ticks of at most two samples per resident
     // 1024-thread CTA (shorter per-sample latency), else two 512-thread CTAs per
@@ -1363,7 +1448,7 @@ struct Problem {
         while (nc < need) nc *= 2;
         if (ovf) E.pool.put(ovf, b_ovf);
         b_ovf = nc * 8;
-        ovf = (uint64_t*)E.pool.get(b_ovf);
+        ovf = (uint64_t*)E.block(E.pool, b_ovf);
         if (!ovf) { ovf_cap = 0; return MANTRA_E_NOMEM; }
         ovf_cap = nc;
         return MANTRA_OK;
@@ -1373,15 +1458,15 @@ struct Problem {
         t0 = now_s();
         const size_t f = std::max<uint32_t>(family(), 1);
         b_hits = f * 8; b_S = (size_t)c * f * (estimator != 0 ? 8 : 4); b_est = f * 8;
-        hits = (u64*)E.pool.get(b_hits);
-        S = (int*)E.pool.get(b_S);
-        est = out_device ? nullptr : (double*)E.pool.get(b_est);
+        hits = (u64*)E.block(E.pool, b_hits);
+        S = (int*)E.block(E.pool, b_S);
+        est = out_device ? nullptr : (double*)E.block(E.pool, b_est);
         if (!hits || !S || (!out_device && !est)) return MANTRA_E_NOMEM;
         CU(cudaMemsetAsync(hits, 0, b_hits, E.sa));
         CU(cudaMemsetAsync(S, 0, b_S, E.sa));
         if (estimator != 0) {
             b_wsq = f * 8;
-            wsq = (u64*)E.pool.get(b_wsq);
+            wsq = (u64*)E.block(E.pool, b_wsq);
             if (!wsq) return MANTRA_E_NOMEM;
             CU(cudaMemsetAsync(wsq, 0, b_wsq, E.sa));
         }
@@ -1809,9 +1894,9 @@ int mantra_graph_load(const uint32_t* u, const uint32_t* v, const uint32_t* t, u
         std::lock_guard<std::mutex> lock(E->mu);
         StoreHost H;
         rc = E->store.build(u, v, t, m, n, &H);
-        if (rc == MANTRA_OK) rc = upload_store(H, G, E->pool, E->sa);
-        if (rc == MANTRA_OK) rc = build_waves(G, E->smem_optin, E->pool, E->sa);
-        if (rc == MANTRA_OK) rc = build_chunks(G, E->smem_optin, E->pool, E->sa);
+        if (rc == MANTRA_OK) rc = upload_store(H, G, *E, E->sa);
+        if (rc == MANTRA_OK) rc = build_waves(G, E->smem_optin, *E, E->sa);
+        if (rc == MANTRA_OK) rc = build_chunks(G, E->smem_optin, *E, E->sa);
         E->store.trim();
     }
     if (rc != MANTRA_OK) { mantra_graph_free(G); return rc; }
@@ -1856,9 +1941,9 @@ void mantra_graph_free(mantra_graph* g) {
         std::lock_guard<std::mutex> lock(E->mu);
         cudaStreamSynchronize(E->sa);
         cudaStreamSynchronize(E->sb);
-        E->pool.put(g->dmem, g->b_dmem);
-        E->pool.put(g->wmem, g->b_wmem);
-        E->pool.put(g->smem, g->b_smem);
+        graph_unblock(*E, g->dmem, g->b_dmem);
+        graph_unblock(*E, g->wmem, g->b_wmem);
+        graph_unblock(*E, g->smem, g->b_smem);
     } else {
         if (g->dmem) cudaFree(g->dmem);
         if (g->wmem) cudaFree(g->wmem);
@@ -1928,7 +2013,7 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
     out->bfs_ms = 1e300;
     for (int nt : {256, 512, 1024})
         for (int sm = 0; sm < 2; ++sm) {
-            if (!E->hop_grid(nt, sm ? g->n : 0, E->hop_regions)) continue;
+            if (!E->hop_grid(nt, sm ? g->n : 0, INT_MAX)) continue;
             Knobs k = none;
             k.bfs_nt = nt; k.bfs_smem = sm;
             double ms = 0;
@@ -2007,7 +2092,7 @@ int stats_run(const mantra_graph* g, mantra_opt opt, uint64_t rs, uint64_t seed,
     const size_t b_cnt = ((size_t)n + 2) * 8;
     const size_t b_clos = clos_out ? al256((size_t)n * 8) : 0;
     const size_t b_all = al256(b_cnt) + 256 + al256(rs * 8) + b_clos;
-    char* blk = (char*)E->pool.get(b_all);
+    char* blk = (char*)E->block(E->pool, b_all);
     if (!blk) return MANTRA_E_NOMEM;
     u64* cnt = (u64*)blk;
     u64* dmax = (u64*)(blk + al256(b_cnt));
@@ -2109,7 +2194,7 @@ int mantra_sample_paths(const mantra_graph* g, mantra_opt opt, uint64_t seed, ui
     std::lock_guard<std::mutex> lock(E->mu);
     const size_t capn = std::max<uint32_t>(cap, 1);
     const size_t bytes = al256(count * 4) * 3 + al256(count * 16) + al256(count * capn * 4) * 2 + al256(count * 8);
-    char* d = (char*)E->pool.get(bytes);
+    char* d = (char*)E->block(E->pool, bytes);
     if (!d) return MANTRA_E_NOMEM;
     std::vector<TickItem> items(1);
     items[0].G = g;

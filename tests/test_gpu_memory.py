@@ -124,3 +124,44 @@ def test_admission_counts_what_is_allocated(M):
     counted, held = map(int, re.search(r"counted (\d+) held (\d+)", r.stdout).groups())
     assert held > 200 << 20                             # the sweep's workspace is part of it
     assert counted >= held - (32 << 20)                 # (tables, captured launches)
+
+
+def test_a_freed_graph_gives_its_memory_back(M):
+    """A large graph's memory is free again after mantra_graph_free; small ones'
+    blocks are kept for the next load, within 256 MB in all."""
+    tri = few_heads(m=6000000)
+    M.Graph(*few_heads(m=70000), n=200).free()
+    before = free_bytes()
+    for _ in range(3):
+        g = M.Graph(*tri, n=200)
+        held = before - free_bytes()
+        assert held > 400 << 20
+        g.free()
+        assert before - free_bytes() <= 260 << 20
+    gs = [M.Graph(*few_heads(m=400000 + k, seed=k), n=200) for k in range(12)]
+    assert before - free_bytes() > 320 << 20
+    for g in gs:
+        g.free()
+    assert before - free_bytes() <= 260 << 20
+
+
+def test_idle_workspaces_make_room(M):
+    """With the device filled, a call that needs more than is left gets the memory of
+    the workspaces that other calls left behind; the results stay the same."""
+    from paper_2304_08356_gb300 import synth
+    big = M.Graph(*synth.chung_lu_bursty(n=20000, m=500000, seed=2))
+    other = M.Graph(*few_heads(), n=200)
+    want = {opt: big.estimate(opt, 0.05, 0.1, 3, fixed_r=2000)[1] for opt in (0, 2, 3)}    # all kernels' workspaces
+    sums = other.estimate(2, 0.05, 0.1, 3, fixed_r=500, target=2)[1]
+    fill = Filler(300 << 20)
+    try:
+        got = other.estimate(2, 0.05, 0.1, 3, fixed_r=500, target=2, c=128)[1]     # 1 GB of Rademacher sums
+        assert np.array_equal(got, sums)
+        for opt in (0, 2, 3):
+            assert np.array_equal(big.estimate(opt, 0.05, 0.1, 3, fixed_r=2000)[1], want[opt])
+    finally:
+        fill.release()
+    for opt in (0, 2, 3):
+        assert np.array_equal(big.estimate(opt, 0.05, 0.1, 3, fixed_r=2000)[1], want[opt])
+    big.free()
+    other.free()
