@@ -332,6 +332,7 @@ struct Engine {
     std::map<uint64_t, int> sc_occ;        // (threads, shared nodes) -> CTAs per SM
     bool tick_n = false;
     bool search_only = false;              // this tick: no room for k_sweep's or k_scan's workspace
+    bool uncapped = false;                 // this tick: only kernels without per-sample caps
     bool tick_b = false, tick_h = false, tick_p = false;   // kernel families with samples in the current tick
     char* pfm_mem = nullptr; PfmWs pws{}; int pfm_grid = 0; uint32_t pfm_n = 0, pfm_lcap = 0; uint64_t pfm_warps = 0;
     // pfm, one CTA per sample: shapes 0 = 256, 1 = 512 threads; modes 0 = state
@@ -1070,14 +1071,15 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     uint32_t nn = 0;
     std::vector<char> sweep(k, 0);
     Engine::SweepPlan plan;
-    const bool sweeps = !wide && !E.search_only && use_sweep(E, items, &plan);
+    const bool streams = !wide && !E.search_only && !E.uncapped, hops = !wide && !E.uncapped;
+    const bool sweeps = streams && use_sweep(E, items, &plan);
     for (uint32_t x = 0; x < k; ++x) {
         const TickItem& it = items[x];
         if (sweeps && can_sweep(it)) {
             sweep[x] = 1;
             any_s = true;
             sunits += (it.job.count + 31) / 32;
-        } else if (!wide && !E.search_only && use_scan(E, it)) {
+        } else if (streams && use_scan(E, it)) {
             sweep[x] = 2;
             any_n = true; nn = std::max(nn, it.G->n);
             nsamples += it.job.count;
@@ -1086,7 +1088,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             pz = std::max(pz, it.G->dg.max_vslots);
             if (!gp || it.G->n > gp->n) gp = it.G;
             pwarps += (it.job.count + 31) / 32;
-        } else if (!wide && on_hop(it.G, it.job)) {
+        } else if (hops && on_hop(it.G, it.job)) {
             any_h = true; hn = std::max(hn, it.G->n); hA = std::max(hA, it.G->A);
             if (!gh || it.G->A > gh->A) gh = it.G;
             hsamples += it.job.count;
@@ -1246,7 +1248,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
             up[np + 1] = up[np] + (cta ? it.job.count : (it.job.count + 31) / 32);
             ++np;
         }
-        else if (!wide && on_hop(it.G, it.job)) { th[nh] = t; uh[nh + 1] = uh[nh] + it.job.count; ++nh; }
+        else if (hops && on_hop(it.G, it.job)) { th[nh] = t; uh[nh + 1] = uh[nh] + it.job.count; ++nh; }
         else { tb[nb] = t; ub[nb + 1] = ub[nb] + it.job.count; ++nb; }
         if (it.reduce) {
             ri[nr] = ReduceItem{it.job.S, it.job.S64, (it.job.ob || it.job.rtb) ? it.job.wsq : it.job.hits, it.job.fam,
@@ -1281,7 +1283,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         else if (items[x].job.opt == MANTRA_PFM)
             log_item(items[x], cta ? "k_pfm_cta" : "k_pfm", wide, cta ? E.tick_pc_nt : 32, cta ? E.tick_pc_sm : 0, c,
                      out->pfm_ms);
-        else if (!wide && on_hop(items[x].G, items[x].job))
+        else if (hops && on_hop(items[x].G, items[x].job))
             log_item(items[x], "k_hop", wide, E.tick_hop_nt, E.tick_hop_sm, c, out->bfs_ms);
         else
             log_item(items[x], "k_bfs", wide, E.tick_bfs_nt, E.tick_bfs_sm, c, out->bfs_ms);
@@ -1289,10 +1291,12 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     return MANTRA_OK;
 }
 
-// A tick followed, for items whose 64-bit path counts overflowed, by a
-// 128-bit re-run of those samples (and their reductions).  counters[x]
-// receives both passes' counters; slot_out[x] the slot whose reduction
-// outputs are current.
+// A tick, followed by re-runs of the samples that it put on the overflow lists:
+// those past a cap of k_hop, k_sweep or k_scan by the 64-bit searches without caps
+// (k_bfs, k_pfm_cta: one sample with long sets is a few milliseconds there, seconds
+// on the stream-scan 128-bit pfm kernel), then those whose path counts passed 64
+// bits by the 128-bit kernels (and their reductions).  tot[x] receives all passes'
+// counters; slot[x] the reduction outputs that are current.
 struct TickResult {
     std::vector<std::vector<char>> slot;   // current reduction outputs per item (copied)
     std::vector<LaunchTotals> tot;         // per item counters, kernel time and launches
@@ -1300,50 +1304,71 @@ struct TickResult {
 };
 
 int run_tick_full(Engine& E, std::vector<TickItem>& items, uint64_t** ovf_lists, TickResult* R) {
-    TickOut out;
-    int rc = run_tick(E, items, false, &out);
-    if (rc != MANTRA_OK) return rc;
     const uint32_t k = (uint32_t)items.size();
     R->slot.assign(k, std::vector<char>(SLOT_BYTES));
     R->tot.assign(k, LaunchTotals());
     R->status.assign(k, MANTRA_OK);
-    std::vector<uint32_t> wide_ix;
-    std::vector<TickItem> witems;
-    for (uint32_t x = 0; x < k; ++x) {
-        std::memcpy(R->slot[x].data(), out.slot[x], SLOT_BYTES);
-        const u64* c = (const u64*)out.slot[x];
-        int st;
-        std::memcpy(&st, out.slot[x] + SLOT_STATUS, 4);
-        R->status[x] = st;
-        R->tot[x].add_counters(c);
-        R->tot[x].launches += 1;
-        R->tot[x].kernel_ms += items[x].job.opt == MANTRA_PFM ? out.pfm_ms : out.bfs_ms;
-        if (st == MANTRA_OK && c[C_NOVF] > 0) {
-            TickItem w = items[x];
-            w.job.idx_list = ovf_lists[x];
-            w.job.count = c[C_NOVF];
-            wide_ix.push_back(x);
-            witems.push_back(w);
-        }
-    }
-    if (!witems.empty()) {
-        TickOut wout;
-        if ((rc = run_tick(E, witems, true, &wout)) != MANTRA_OK) return rc;
-        for (size_t y = 0; y < witems.size(); ++y) {
-            const uint32_t x = wide_ix[y];
-            const u64* c = (const u64*)wout.slot[y];
+    // a pass over items of the tick (ix: whose), its results added to theirs
+    auto pass = [&](std::vector<TickItem>& its, const std::vector<uint32_t>& ix, bool wide, std::vector<u64>* novf,
+                    std::vector<u64>* ncap) -> int {
+        TickOut out;
+        const int rc = run_tick(E, its, wide, &out);
+        if (rc != MANTRA_OK) return rc;
+        for (size_t y = 0; y < its.size(); ++y) {
+            const uint32_t x = ix[y];
+            const u64* c = (const u64*)out.slot[y];
             int st;
-            std::memcpy(&st, wout.slot[y] + SLOT_STATUS, 4);
+            std::memcpy(&st, out.slot[y] + SLOT_STATUS, 4);
             if (st != MANTRA_OK) R->status[x] = st;
             R->tot[x].add_counters(c);
             R->tot[x].launches += 1;
-            R->tot[x].wide += witems[y].job.count;
-            R->tot[x].kernel_ms += witems[y].job.opt == MANTRA_PFM ? wout.pfm_ms : wout.bfs_ms;
-            // reduction outputs of the wide tick include every sample of the round
-            std::memcpy(R->slot[x].data() + SLOT_HMAX, wout.slot[y] + SLOT_HMAX, SLOT_BYTES - SLOT_HMAX);
+            if (wide) R->tot[x].wide += its[y].job.count;
+            R->tot[x].kernel_ms += its[y].job.opt == MANTRA_PFM ? out.pfm_ms : out.bfs_ms;
+            // reduction outputs of a later pass include every sample of the round
+            std::memcpy(R->slot[x].data() + SLOT_HMAX, out.slot[y] + SLOT_HMAX, SLOT_BYTES - SLOT_HMAX);
+            if (novf) novf->push_back(st == MANTRA_OK ? c[C_NOVF] : 0);
+            if (ncap) ncap->push_back(st == MANTRA_OK ? c[C_NCAP] : 0);
+        }
+        return MANTRA_OK;
+    };
+    auto listed = [&](uint32_t x, uint64_t* list, u64 count) {
+        TickItem w = items[x];
+        w.job.idx_list = list;
+        w.job.count = count;
+        return w;
+    };
+    std::vector<uint32_t> all(k), cix, wix;
+    for (uint32_t x = 0; x < k; ++x) all[x] = x;
+    std::vector<u64> novf, ncap;
+    int rc = pass(items, all, false, &novf, &ncap);
+    if (rc != MANTRA_OK) return rc;
+    std::vector<TickItem> citems, witems;
+    std::vector<std::pair<void*, size_t>> lists;   // overflow lists of the second pass
+    for (uint32_t x = 0; x < k; ++x) {
+        if (novf[x]) { wix.push_back(x); witems.push_back(listed(x, ovf_lists[x], novf[x])); }
+        if (!ncap[x]) continue;
+        TickItem c = listed(x, ovf_lists[x] + (items[x].job.count - ncap[x]), ncap[x]);
+        c.job.ovf_list = (uint64_t*)E.block(E.pool, ncap[x] * 8, true);
+        if (c.job.ovf_list) {
+            lists.emplace_back(c.job.ovf_list, ncap[x] * 8);
+            cix.push_back(x);
+            citems.push_back(c);
+        } else {                                   // no room for a list: the 128-bit kernels take them
+            wix.push_back(x);
+            witems.push_back(c);
         }
     }
-    return MANTRA_OK;
+    if (!citems.empty()) {
+        novf.clear();
+        E.uncapped = true;
+        rc = pass(citems, cix, false, &novf, nullptr);
+        E.uncapped = false;
+        for (size_t y = 0; rc == MANTRA_OK && y < citems.size(); ++y)
+            if (novf[y]) { wix.push_back(cix[y]); witems.push_back(listed(cix[y], citems[y].job.ovf_list, novf[y])); }
+    }
+    if (rc == MANTRA_OK && !witems.empty()) rc = pass(witems, wix, true, nullptr, nullptr);
+    for (auto& l : lists) E.pool.put(l.first, l.second);
+    return rc;
 }
 
 // Theorem 1 (supremum-deviation bound) pieces, natural logarithms.

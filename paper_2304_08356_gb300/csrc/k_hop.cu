@@ -377,8 +377,8 @@ __device__ __forceinline__ bool hop_small(const HopWs& ws, uint32_t k, uint32_t 
 // After the levels of a sample, all threads of the CTA: with z found from level
 // k (events [q0, q1)), the states on optimal paths, their counts, the draw (or
 // the ob values), then the sample's hits, Rademacher sums and record.  E0: the
-// sample's first level stamp.  Sets S.ovf when the sample
-// needs the 128-bit kernel.  Out of line, so that the levels' loop does not
+// sample's first level stamp.  Sets S.ovf to 1 when the sample needs the 128-bit
+// kernel, to 2 when it exceeds a cap.  Out of line, so that the levels' loop does not
 // carry its registers.
 template <int NT>
 __device__ __noinline__ void hop_finish(const HopWs* wsp, bool found, uint32_t k, uint32_t q0, uint32_t q1,
@@ -448,7 +448,7 @@ __device__ __noinline__ void hop_finish(const HopWs* wsp, bool found, uint32_t k
             Gw[0] = z; Gs[0] = 0; Gs[1] = nC;
             clev[d] = 0; clev[d - 1] = nC; glev[d] = 0; glev[d - 1] = 1;
         }
-        if (nC > ws.c_cap) S.ovf = 1u;
+        if (nC > ws.c_cap) S.ovf = 2u;
         // level lv - 1 from level lv
         uint32_t cb = 0;                     // first state of level lv
         for (uint32_t lv = d; lv >= 2 && nC <= ws.c_cap; --lv) {
@@ -598,7 +598,7 @@ __device__ __noinline__ void hop_finish(const HopWs* wsp, bool found, uint32_t k
                 Gs[ng] = nC;
                 clev[lv - 2] = nC;
                 glev[lv - 2] = ng;
-                if (nC > ws.c_cap) S.ovf = 1u;
+                if (nC > ws.c_cap) S.ovf = 2u;
             }
         }
         __syncthreads();
@@ -740,8 +740,10 @@ __device__ __noinline__ void hop_finish(const HopWs* wsp, bool found, uint32_t k
     __syncthreads();
 
     if (S.ovf) {
-        // the 128-bit re-run takes (and counts) the sample
-        if (tid == 0) push_overflow(job, i);
+        // another kernel takes (and counts) the sample
+        if (tid == 0) {
+            if (S.ovf == 2u) push_capped(job, i); else push_overflow(job, i);
+        }
     } else {
         if (!S.err && !job.stats) {
             const uint32_t nint = family_count(job, S.len);
@@ -1132,7 +1134,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_hop(const Task* tasks, const 
                     for (int x = 0; x < WALK_K; ++x)
                         if (was[x] == 0u) {                  // a first touch
                             const uint32_t p = atomicAdd(S.nq + nx, 1u);
-                            if (p < cap) Qn[p] = v[x]; else S.ovf = 1u;
+                            if (p < cap) Qn[p] = v[x]; else S.ovf = 2u;
                         }
                 });
                 __syncthreads();
@@ -1168,16 +1170,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_hop(const Task* tasks, const 
 
 // Host-side launch helpers -------------------------------------------------
 
-// Region of one CTA.  Events per sample are capped at A / 4 + 2 n + 4096 (a
-// search of the bursty graphs makes one event per five states) and the states
+// Region of one CTA.  Above 2^18 slots (where a region would grow from 10 to 19
+// bytes a slot) the events of a sample are capped at A / 4 + 2 n + 4096 (a
+// search of the bursty graphs makes one event per five states), and the states
 // on optimal paths at A / 8 + 65536 (they are a few hundred at most there);
-// a sample that needs more goes to the 128-bit kernel, which has no such cap.
+// a sample that needs more goes to k_bfs, which has no such cap.
 size_t hop_region_bytes(uint32_t n, uint32_t A, HopWs* ws) {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const uint64_t all = (uint64_t)A + 1;
     ws->n_cap = n;
     ws->A_cap = A;
-    ws->ev_cap = (uint32_t)std::min<uint64_t>(all, (uint64_t)A / 4 + 2ull * n + 4096);
+    ws->ev_cap = (uint32_t)(A <= 1u << 18 ? all : std::min<uint64_t>(all, (uint64_t)A / 4 + 2ull * n + 4096));
     ws->c_cap = (uint32_t)std::min<uint64_t>(all, (uint64_t)A / 8 + 65536);
     const size_t nq = std::max<size_t>(ws->ev_cap, 2 * (size_t)n), ng = (size_t)ws->c_cap + n + 4;
     size_t o = 0;

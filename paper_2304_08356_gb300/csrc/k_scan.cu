@@ -255,7 +255,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_scan(const Task* tasks, const
             if (reached) {
                 // the way back: path[k], edge into it pathe[k]
                 uint32_t v = z, plen = 0;
-                bool choice = false, bad = false, perr = false;
+                bool choice = false, perr = false;
+                uint32_t away = 0;                           // CHOICE_OVF or CHOICE_CAPPED
                 u64 tot = 1;                                 // the only path: nothing to draw
                 while (v != s) {
                     const uint32_t a = arr[v], e0 = g.slot_in[a], e1 = g.slot_in[a + 1];
@@ -283,121 +284,15 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_scan(const Task* tasks, const
                 }
                 __syncwarp();
                 if (choice) {
-                    if (lane == 0) {
-                        S.cnt = 1;
-                        cv[0] = z;
-                        MK[z >> 5] |= 1u << (z & 31u);
-                    }
-                    __syncwarp();
-                    uint32_t cnt = 1;
-                    for (uint32_t h = 0; h < cnt;) {
-                        const uint32_t p = h + lane;
-                        if (p < cnt) {
-                            const uint32_t v = cv[p];
-                            if (v != s) {
-                                const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                                for (uint32_t e = g.slot_in[a]; e < e1; ++e) {
-                                    const uint32_t w = g.in_u[e];
-                                    if (!before(w, tv)) continue;
-                                    if (atomicOr(MK + (w >> 5), 1u << (w & 31u)) & (1u << (w & 31u))) continue;
-                                    const uint32_t x = atomicAdd(&S.cnt, 1u);
-                                    cv[x] = w;
-                                }
-                            }
-                        }
-                        __syncwarp();
-                        h = min(h + 32u, cnt);
-                        cnt = S.cnt;
-                        __syncwarp();
-                    }
-                    for (uint32_t p = lane; p < cnt; p += 32) MK[cv[p] >> 5] = 0u;
-                    __syncwarp();
-                    if (!bad) {
-                        // by arrival time (s first); a vertex's in-edges come from earlier arrivals
-                        for (uint32_t p = lane; p < cnt; p += 32) {
-                            const uint32_t v = cv[p];
-                            ck[p] = v == s ? 0ull : ((u64)(g.slot_t[arr[v]] + 1u) << 32 | v);
-                        }
-                        __syncwarp();
-                        for (uint32_t p = lane; p < cnt; p += 32) {
-                            const u64 kv = ck[p];
-                            uint32_t r = 0;
-                            for (uint32_t y = 0; y < cnt; ++y) r += ck[y] < kv ? 1u : 0u;
-                            co[r] = cv[p];
-                        }
-                        __syncwarp();
-                        for (uint32_t p = 0; p < cnt && !bad; ++p) {
-                            const uint32_t v = co[p];
-                            u64 sum = 0;
-                            bool wrap = false;
-                            if (v == s) {
-                                sum = lane == 0 ? 1ull : 0ull;
-                            } else {
-                                const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                                for (uint32_t e = g.slot_in[a] + lane; e < e1; e += 32) {
-                                    const uint32_t w = g.in_u[e];
-                                    if (!before(w, tv)) continue;
-                                    const u64 y = sum + sig[w];
-                                    wrap |= y < sum;
-                                    sum = y;
-                                }
-                            }
-        #pragma unroll
-                            for (int o = 16; o > 0; o >>= 1) {
-                                const u64 y = shfl_xor_w(sum, o), y2 = sum + y;
-                                wrap |= y2 < sum;
-                                sum = y2;
-                            }
-                            bad = __any_sync(FULL, wrap);
-                            if (lane == 0) sig[v] = sum;
-                            __syncwarp();
-                            tot = sum;                               // the last one is z (the latest arrival)
-                        }
-                    }
-                    plen = 0;
-                    if (!bad) {
-                        tot = sig[z];
-                        u128 x = 0;
-                        uint32_t ok = 1;
-                        if (lane == 0) ok = draw_below128((u128)tot, job.seed, i, job.dom_path, &x) ? 1u : 0u;
-                        ok = __shfl_sync(FULL, ok, 0);
-                        u64 xs = shfl_idx_w((u64)x, 0);
-                        if (!ok) { perr = true; if (lane == 0) set_status(job.status, ST_RNG); }
-                        v = z;
-                        while (!perr && !bad && v != s) {
-                            const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                            uint32_t nxt = NONE, ech = 0;
-                            for (uint32_t e0 = g.slot_in[a]; e0 < e1; e0 += 32) {
-                                const uint32_t e = e0 + lane;
-                                u64 wt = 0;
-                                uint32_t w = 0;
-                                if (e < e1) {
-                                    w = g.in_u[e];
-                                    if (before(w, tv)) wt = sig[w];
-                                }
-                                const u64 incl = warp_inclusive_sum(wt);
-                                const unsigned msk = __ballot_sync(FULL, xs < incl);
-                                if (msk) {
-                                    const int l = __ffs(msk) - 1;
-                                    nxt = __shfl_sync(FULL, w, l);
-                                    ech = e0 + l;
-                                    xs -= shfl_idx_w(incl - wt, l);
-                                    break;
-                                }
-                                xs -= shfl_idx_w(incl, 31);
-                            }
-                            if (nxt == NONE || plen > n) { perr = true; break; }
-                            if (lane == 0) { path[plen] = v; pathe[plen] = ech; }
-                            ++plen;
-                            v = nxt;
-                        }
-                        if (lane == 0 && !perr && !bad) path[plen] = s;
-                        ++plen;
-                    }
+                    const int got = draw_choice(g, job, i, s, z, arr, before,
+                                                ChoiceWs{cv, co, ck, sig, MK, ws.cone_cap, n + 2u}, &S.cnt, path, pathe,
+                                                &plen, &tot);
+                    perr = got == CHOICE_ERR;
+                    away = got == CHOICE_OVF || got == CHOICE_CAPPED ? (uint32_t)got : 0u;
                 }
                 if (lane == 0) {
                     if (perr) { S.err = 1; set_status(job.status, ST_CHECK); }
-                    else if (bad) S.ovf = 1;
+                    else if (away) S.ovf = away;
                     else {
                         S.len = plen;
                         S.sigma = tot;
@@ -410,8 +305,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_scan(const Task* tasks, const
         }
         __syncthreads();
         if (S.ovf) {
-            // the 128-bit kernel takes (and counts) the sample
-            if (tid == 0) push_overflow(job, i);
+            // another kernel takes (and counts) the sample
+            if (tid == 0) {
+                if (S.ovf == CHOICE_CAPPED) push_capped(job, i); else push_overflow(job, i);
+            }
             for (uint32_t v = tid; v < n; v += NT) {
                 if (v == s || !((FB[v >> 5] >> (v & 31u)) & 1u)) continue;
                 const uint32_t a = arr[v], tv = g.slot_t[a];
@@ -463,13 +360,14 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_scan(const Task* tasks, const
 
 size_t scan_region_bytes(uint32_t n, ScanWs* ws) {
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    ws->cone_cap = std::min<uint32_t>(n + 1, 2048);
     size_t o = 0;
     ws->o_arr = o;   o = al(o + (size_t)n * 4);
     ws->o_path = o;  o = al(o + (size_t)(n + 2) * 4);
     ws->o_pathe = o; o = al(o + (size_t)(n + 2) * 4);
-    ws->o_cv = o;    o = al(o + (size_t)n * 4);
-    ws->o_co = o;    o = al(o + (size_t)n * 4);
-    ws->o_ck = o;    o = al(o + (size_t)n * 8);
+    ws->o_cv = o;    o = al(o + (size_t)ws->cone_cap * 4);
+    ws->o_co = o;    o = al(o + (size_t)ws->cone_cap * 4);
+    ws->o_ck = o;    o = al(o + (size_t)ws->cone_cap * 8);
     ws->o_sig = o;   o = al(o + (size_t)n * 8);
     ws->o_mk = o;    o = al(o + (size_t)((n + 31) / 32) * 4);
     return o;

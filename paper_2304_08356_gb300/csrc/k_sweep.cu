@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
         }
         // ---- backward from z through the log, all samples together ----
         uint32_t len = 0;                                    // path vertices
-        bool choice = false, ovf = false, err = false;
+        bool choice = false, ovf = false, capped = false, err = false;
         u64 sigma = 0;
         {
             uint32_t cur = reached ? z : NONE;               // the path's vertex whose record is wanted
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
                     if (at) {
                         const uint32_t a = __ldg(g.wave_at + pos).x, e0 = g.slot_in[a];
                         if (g.slot_in[a + 1] - e0 > 1u) { choice = true; cur = NONE; }
-                        else if (len + 2 > ws.path_cap) { ovf = true; cur = NONE; }
+                        else if (len + 2 > ws.path_cap) { capped = true; cur = NONE; }
                         else {
                             pv[len] = v; pe[len] = e0;
                             ++len;
@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
             for (uint32_t x = lane; x < bw; x += 32) WM[x] = 0u;
             __syncwarp();
         }
-        if (choice || ovf) len = 0;
+        if (choice || capped) len = 0;
         // fa(w) < tv for the sample whose arrivals are in arr, with source src
         auto fa_before = [&](uint32_t w, uint32_t src, uint32_t j, uint32_t tv) -> bool {
             if (w == src) return true;
@@ -347,139 +347,29 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
             const uint32_t sj = __shfl_sync(FULL, s, j), zj = __shfl_sync(FULL, z, j);
             const uint64_t ij = __shfl_sync(FULL, i, j);
             copy_arrivals(j);
-            if (lane == 0) {
-                sh_cnt = 1;
-                cv[0] = zj;
-                MK[zj >> 5] |= 1u << (zj & 31u);
-            }
-            __syncwarp();
-            uint32_t cnt = 1;
-            for (uint32_t h = 0; h < cnt && cnt <= ws.cone_cap;) {
-                const uint32_t p = h + lane;
-                if (p < cnt) {
-                    const uint32_t v = cv[p];
-                    if (v != sj) {
-                        const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                        for (uint32_t e = g.slot_in[a]; e < e1; ++e) {
-                            const uint32_t w = g.in_u[e];
-                            if (!fa_before(w, sj, j, tv)) continue;
-                            if (atomicOr(MK + (w >> 5), 1u << (w & 31u)) & (1u << (w & 31u))) continue;
-                            const uint32_t x = atomicAdd(&sh_cnt, 1u);
-                            if (x < ws.cone_cap) cv[x] = w;
-                            else atomicAnd(MK + (w >> 5), ~(1u << (w & 31u)));
-                        }
-                    }
-                }
-                __syncwarp();
-                h = min(h + 32u, cnt);
-                cnt = sh_cnt;
-                __syncwarp();
-            }
-            const uint32_t got = min(cnt, ws.cone_cap);
-            bool bad = cnt > ws.cone_cap;
-            for (uint32_t p = lane; p < got; p += 32) MK[cv[p] >> 5] = 0u;
-            __syncwarp();
-            u64 tot = 0;
-            if (!bad) {
-                // by arrival time (s first); a vertex's in-edges come from earlier arrivals
-                for (uint32_t p = lane; p < cnt; p += 32) {
-                    const uint32_t v = cv[p];
-                    ck[p] = v == sj ? 0ull : ((u64)(g.slot_t[arr[v]] + 1u) << 32 | v);
-                }
-                __syncwarp();
-                for (uint32_t p = lane; p < cnt; p += 32) {
-                    const u64 kv = ck[p];
-                    uint32_t r = 0;
-                    for (uint32_t y = 0; y < cnt; ++y) r += ck[y] < kv ? 1u : 0u;
-                    co[r] = cv[p];
-                }
-                __syncwarp();
-                for (uint32_t p = 0; p < cnt && !bad; ++p) {
-                    const uint32_t v = co[p];
-                    u64 sum = 0;
-                    bool wrap = false;
-                    if (v == sj) {
-                        sum = lane == 0 ? 1ull : 0ull;
-                    } else {
-                        const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                        for (uint32_t e = g.slot_in[a] + lane; e < e1; e += 32) {
-                            const uint32_t w = g.in_u[e];
-                            if (!fa_before(w, sj, j, tv)) continue;
-                            const u64 y = sum + sig[w];
-                            wrap |= y < sum;
-                            sum = y;
-                        }
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        const u64 y = shfl_xor_w(sum, o), z2 = sum + y;
-                        wrap |= z2 < sum;
-                        sum = z2;
-                    }
-                    bad = __any_sync(FULL, wrap);
-                    if (lane == 0) sig[v] = sum;
-                    __syncwarp();
-                    tot = sum;                               // the last one is z (the latest arrival)
-                }
-            }
             uint32_t plen = 0;
-            bool perr = false;
-            if (!bad) {
-                tot = sig[zj];
-                u128 x = 0;
-                uint32_t ok = 1;
-                if (lane == 0) ok = draw_below128((u128)tot, job.seed, ij, job.dom_path, &x) ? 1u : 0u;
-                ok = __shfl_sync(FULL, ok, 0);
-                u64 xs = shfl_idx_w((u64)x, 0);
-                if (!ok) { perr = true; if (lane == 0) set_status(job.status, ST_RNG); }
-                uint32_t v = zj;
-                while (!perr && !bad && v != sj) {
-                    if (plen + 2 > ws.path_cap) { bad = true; break; }
-                    const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
-                    uint32_t nxt = NONE, ech = 0;
-                    for (uint32_t e0 = g.slot_in[a]; e0 < e1; e0 += 32) {
-                        const uint32_t e = e0 + lane;
-                        u64 wt = 0;
-                        uint32_t w = 0;
-                        if (e < e1) {
-                            w = g.in_u[e];
-                            if (fa_before(w, sj, j, tv)) wt = sig[w];
-                        }
-                        const u64 incl = warp_inclusive_sum(wt);
-                        const unsigned msk = __ballot_sync(FULL, xs < incl);
-                        if (msk) {
-                            const int l = __ffs(msk) - 1;
-                            nxt = __shfl_sync(FULL, w, l);
-                            ech = e0 + l;
-                            xs -= shfl_idx_w(incl - wt, l);
-                            break;
-                        }
-                        xs -= shfl_idx_w(incl, 31);
-                    }
-                    if (nxt == NONE || plen > n) { perr = true; break; }
-                    if (lane == 0) { path[(size_t)j * ws.path_cap + plen] = v; pathe[(size_t)j * ws.path_cap + plen] = ech; }
-                    ++plen;
-                    v = nxt;
-                }
-                if (lane == 0 && !perr && !bad) path[(size_t)j * ws.path_cap + plen] = sj;
-                ++plen;
-            }
+            u64 tot = 0;
+            const int got = draw_choice(g, job, ij, sj, zj, arr, [&](uint32_t w, uint32_t tv) { return fa_before(w, sj, j, tv); },
+                                        ChoiceWs{cv, co, ck, sig, MK, ws.cone_cap, ws.path_cap}, &sh_cnt,
+                                        path + (size_t)j * ws.path_cap, pathe + (size_t)j * ws.path_cap, &plen, &tot);
             if (lane == j) {
                 choice = false;
-                if (bad) ovf = true;
-                else if (perr) err = true;
-                else { len = plen; sigma = tot; }
+                ovf = got == CHOICE_OVF;
+                capped = got == CHOICE_CAPPED;
+                err = got == CHOICE_ERR;
+                if (got == CHOICE_DRAWN) { len = plen; sigma = tot; }
             }
             __syncwarp();
         }
         if (err) set_status(job.status, ST_CHECK);
         if (ovf) push_overflow(job, i);
+        if (capped) push_capped(job, i);
         // ---- hits, Rademacher sums and records, a sample at a time ----
         uint32_t rade[4] = {0, 0, 0, 0};
         if (len > 0) philox_block(job.seed, i, DOM_RADE, 0, rade);
         u64 c_int = 0;
         __syncwarp();
-        for (unsigned todo = __ballot_sync(FULL, have && !ovf && !err && (len > 0 || job.rec_len)); todo; todo &= todo - 1) {
+        for (unsigned todo = __ballot_sync(FULL, have && !ovf && !capped && !err && (len > 0 || job.rec_len)); todo; todo &= todo - 1) {
             const uint32_t j = __ffs(todo) - 1;
             const uint32_t lj = __shfl_sync(FULL, len, j);
             const uint32_t nint = job.target == 0 ? (lj < 2 ? 0u : lj - 2u) : (lj < 2 ? 0u : lj - 1u);
@@ -519,8 +409,8 @@ __global__ void __launch_bounds__(32) k_sweep(const Task* tasks, const uint64_t*
                         job.rec_edges[r * job.rec_cap + p] = pe[lj - 2 - p];
             }
         }
-        // ---- counters; a sample that the 128-bit kernel re-runs is counted there ----
-        for (unsigned todo = __ballot_sync(FULL, ovf); todo; todo &= todo - 1) {
+        // ---- counters; a sample that another kernel re-runs is counted there ----
+        for (unsigned todo = __ballot_sync(FULL, ovf || capped); todo; todo &= todo - 1) {
             const uint32_t j = __ffs(todo) - 1, sj = __shfl_sync(FULL, s, j), tej = __shfl_sync(FULL, te, j);
             copy_arrivals(j);
             if (lane == j) c_scan = 0;

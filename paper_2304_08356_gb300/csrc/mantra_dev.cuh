@@ -31,10 +31,11 @@ constexpr uint32_t NONE = 0xFFFFFFFFu;
 enum : int { ST_OK = 0, ST_OVERFLOW = 3, ST_TIMEOUT = 5, ST_CHECK = 6, ST_RNG = 7 };
 
 // Counter slots of a launch (u64 each).
+// C_NOVF, C_NCAP: entries of the overflow list from its front and from its back.
 // C_FSEG: sh/sfm frontier vertices; CTA pfm kernel: frontier rounds.
 // C_XEDGE: CTA pfm kernel, out-edges of the arrival expansions plus the DAG
 // edges of the Kahn pass; diagnostics only.
-enum : int { C_WORK = 0, C_SUMINT = 1, C_ESCAN = 2, C_EADD = 3, C_SNEW = 4, C_NOVF = 5, C_FSEG = 6, C_XEDGE = 7,
+enum : int { C_NCAP = 0, C_SUMINT = 1, C_ESCAN = 2, C_EADD = 3, C_SNEW = 4, C_NOVF = 5, C_FSEG = 6, C_XEDGE = 7,
              C_NCOUNT = 8 };
 
 struct DevGraph {
@@ -126,7 +127,8 @@ struct Job {
     u64* wsq;                  // F (ob, RTB)
     long long* S64;            // c*F (ob, RTB), or nullptr
     u64* ctr;                  // C_NCOUNT counters
-    uint64_t* ovf_list;        // sample indices whose 64-bit path counts overflowed
+    uint64_t* ovf_list;        // count entries: from the front the samples whose 64-bit path counts overflowed,
+                               // from the back those that a kernel with per-sample caps could not hold
     int* status;
     // optional per-sample records, indexed by (sample index - i0)
     uint32_t* rec_s;
@@ -754,6 +756,154 @@ __device__ __forceinline__ void push_overflow(const Job& job, uint64_t i) {
     else set_status(job.status, ST_CHECK);
 }
 
+// A sample that exceeds a per-sample cap of k_hop, k_sweep or k_scan: the 64-bit
+// search without caps (k_bfs, k_pfm_cta) takes it.
+__device__ __forceinline__ void push_capped(const Job& job, uint64_t i) {
+    if (job.ovf_list) job.ovf_list[job.count - 1ull - atomicAdd(job.ctr + C_NCAP, 1ull)] = i;
+    else set_status(job.status, ST_CHECK);
+}
+
+// ---- pfm samples whose way back has a choice (k_sweep, k_scan) ----
+
+// Scratch of draw_choice: the vertices that lead to z, the same by arrival time and
+// their sort keys (cap each), their path counts by vertex, a mark per vertex (0
+// between uses).
+struct ChoiceWs {
+    uint32_t *cv, *co;
+    u64 *ck, *sig;
+    uint32_t* marks;
+    uint32_t cap, path_cap;
+};
+
+enum : int { CHOICE_DRAWN = 0, CHOICE_OVF = 1, CHOICE_CAPPED = 2, CHOICE_ERR = 3 };
+
+// By one warp: the vertices that lead from s to z over prefix-foremost in-edges,
+// their path counts and the drawn path (path[k] from z, pathe[k] the in-CSR index
+// of the edge into it).  arr[v]: v's arrival slot; before(w, tv): w was reached
+// before tv; cnt: a word of shared memory.  CHOICE_OVF: a count passes 64 bits;
+// CHOICE_CAPPED: more vertices than cap, or path_cap.  The ranks take cap^2 / 32
+// steps and the counts a chain of loads per vertex, hence the caps.
+template <class Before>
+__device__ __forceinline__ int draw_choice(const DevGraph& g, const Job& job, uint64_t i, uint32_t s, uint32_t z,
+                                           const uint32_t* arr, Before before, const ChoiceWs& c, uint32_t* cnt_sh,
+                                           uint32_t* path, uint32_t* pathe, uint32_t* plen_out, u64* tot_out) {
+    constexpr uint32_t FULL = 0xFFFFFFFFu;
+    const uint32_t lane = threadIdx.x & 31;
+    if (lane == 0) {
+        *cnt_sh = 1;
+        c.cv[0] = z;
+        c.marks[z >> 5] |= 1u << (z & 31u);
+    }
+    __syncwarp();
+    uint32_t cnt = 1;
+    for (uint32_t h = 0; h < cnt && cnt <= c.cap;) {
+        const uint32_t p = h + lane;
+        if (p < cnt) {
+            const uint32_t v = c.cv[p];
+            if (v != s) {
+                const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
+                for (uint32_t e = g.slot_in[a]; e < e1; ++e) {
+                    const uint32_t w = g.in_u[e];
+                    if (!before(w, tv)) continue;
+                    if (atomicOr(c.marks + (w >> 5), 1u << (w & 31u)) & (1u << (w & 31u))) continue;
+                    const uint32_t x = atomicAdd(cnt_sh, 1u);
+                    if (x < c.cap) c.cv[x] = w;
+                    else atomicAnd(c.marks + (w >> 5), ~(1u << (w & 31u)));
+                }
+            }
+        }
+        __syncwarp();
+        h = min(h + 32u, cnt);
+        cnt = *cnt_sh;
+        __syncwarp();
+    }
+    for (uint32_t p = lane; p < min(cnt, c.cap); p += 32) c.marks[c.cv[p] >> 5] = 0u;
+    __syncwarp();
+    if (cnt > c.cap) return CHOICE_CAPPED;
+    // by arrival time (s first); a vertex's in-edges come from earlier arrivals
+    for (uint32_t p = lane; p < cnt; p += 32) {
+        const uint32_t v = c.cv[p];
+        c.ck[p] = v == s ? 0ull : ((u64)(g.slot_t[arr[v]] + 1u) << 32 | v);
+    }
+    __syncwarp();
+    for (uint32_t p = lane; p < cnt; p += 32) {
+        const u64 kv = c.ck[p];
+        uint32_t r = 0;
+        for (uint32_t y = 0; y < cnt; ++y) r += c.ck[y] < kv ? 1u : 0u;
+        c.co[r] = c.cv[p];
+    }
+    __syncwarp();
+    for (uint32_t p = 0; p < cnt; ++p) {
+        const uint32_t v = c.co[p];
+        u64 sum = 0;
+        bool wrap = false;
+        if (v == s) {
+            sum = lane == 0 ? 1ull : 0ull;
+        } else {
+            const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
+            for (uint32_t e = g.slot_in[a] + lane; e < e1; e += 32) {
+                const uint32_t w = g.in_u[e];
+                if (!before(w, tv)) continue;
+                const u64 y = sum + c.sig[w];
+                wrap |= y < sum;
+                sum = y;
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const u64 y = shfl_xor_w(sum, o), y2 = sum + y;
+            wrap |= y2 < sum;
+            sum = y2;
+        }
+        if (__any_sync(FULL, wrap)) return CHOICE_OVF;
+        if (lane == 0) c.sig[v] = sum;
+        __syncwarp();
+    }
+    const u64 tot = c.sig[z];
+    u128 x = 0;
+    uint32_t ok = 1;
+    if (lane == 0) ok = draw_below128((u128)tot, job.seed, i, job.dom_path, &x) ? 1u : 0u;
+    ok = __shfl_sync(FULL, ok, 0);
+    u64 xs = shfl_idx_w((u64)x, 0);
+    if (!ok) {
+        if (lane == 0) set_status(job.status, ST_RNG);
+        return CHOICE_ERR;
+    }
+    uint32_t v = z, plen = 0;
+    while (v != s) {
+        if (plen + 2 > c.path_cap) return CHOICE_CAPPED;
+        const uint32_t a = arr[v], tv = g.slot_t[a], e1 = g.slot_in[a + 1];
+        uint32_t nxt = NONE, ech = 0;
+        for (uint32_t e0 = g.slot_in[a]; e0 < e1; e0 += 32) {
+            const uint32_t e = e0 + lane;
+            u64 wt = 0;
+            uint32_t w = 0;
+            if (e < e1) {
+                w = g.in_u[e];
+                if (before(w, tv)) wt = c.sig[w];
+            }
+            const u64 incl = warp_inclusive_sum(wt);
+            const unsigned msk = __ballot_sync(FULL, xs < incl);
+            if (msk) {
+                const int l = __ffs(msk) - 1;
+                nxt = __shfl_sync(FULL, w, l);
+                ech = e0 + l;
+                xs -= shfl_idx_w(incl - wt, l);
+                break;
+            }
+            xs -= shfl_idx_w(incl, 31);
+        }
+        if (nxt == NONE) return CHOICE_ERR;
+        if (lane == 0) { path[plen] = v; pathe[plen] = ech; }
+        ++plen;
+        v = nxt;
+    }
+    if (lane == 0) path[plen] = s;
+    *plen_out = plen + 1u;
+    *tot_out = tot;
+    return CHOICE_DRAWN;
+}
+
 // Entries of the estimated family that a drawn path of len vertices adds one
 // hit to: its len-2 internal vertices (Sec. 3) or its len-1 edges (App. A).
 __device__ __forceinline__ uint32_t family_count(const Job& job, uint32_t len) {
@@ -794,8 +944,8 @@ struct HopWs {
            o_path, o_pathe, o_stamp;
     uint32_t n_cap;      // node capacity of a region
     uint32_t A_cap;      // slot capacity of a region
-    uint32_t ev_cap;     // (vertex, level) events per sample; more: the sample goes to the overflow list
-    uint32_t c_cap;      // states on optimal paths per sample; more: the overflow list
+    uint32_t ev_cap;     // (vertex, level) events per sample; more: push_capped
+    uint32_t c_cap;      // states on optimal paths per sample; more: push_capped
     int nt;              // threads per CTA (256, 512 or 1024)
     uint32_t n_smem;     // nodes whose next-level arrivals are in dynamic shared memory (0: in the region)
 };
@@ -805,6 +955,7 @@ struct ScanWs {
     char* base;          // CTA b uses base + b * stride
     size_t stride;
     size_t o_arr, o_path, o_pathe, o_cv, o_co, o_ck, o_sig, o_mk;
+    uint32_t cone_cap;   // vertices that lead to z of a sample with a choice; more: push_capped
     uint32_t n_smem;     // nodes of the shared-memory bits
     int nt;              // threads per CTA (512 or 1024)
 };
@@ -816,8 +967,8 @@ struct SweepWs {
     size_t o_log, o_arr, o_stp, o_path, o_pathe, o_cv, o_co, o_ck, o_sig;
     uint32_t* order;     // or nullptr: the units' samples (32 places per unit), see k_sweep_order
     uint32_t n_smem;     // nodes of the shared-memory state
-    uint32_t path_cap;   // vertices of a path; longer: the sample goes to the overflow list
-    uint32_t cone_cap;   // vertices that lead to z of a sample with a choice; more: the overflow list
+    uint32_t path_cap;   // vertices of a path; longer: push_capped
+    uint32_t cone_cap;   // vertices that lead to z of a sample with a choice; more: push_capped
 };
 
 // Per-warp scratch of the pfm search kernel.
