@@ -63,8 +63,17 @@ int main() {
     a = small.get(512);
     b = small.get(700);
     small.put(a, 512);
-    small.put(b, 700);                          // 512 + 768 exceeds it: given back at once
-    CHECK(small.cached == 512 && g_left == 4096 - 512);
+    small.put(b, 700);                          // 512 + 768 exceeds it: the older block goes
+    CHECK(small.cached == 768 && g_left == 4096 - 768 && small.get(768) == b);
+    small.put(b, 768);
+    a = small.get(2048);
+    small.put(a, 2048);                         // larger than the cache may be
+    CHECK(small.cached == 768 && g_left == 4096 - 768);
+    a = small.get(256);
+    small.put(a, 256);                          // both fit
+    CHECK(small.cached == 1024 && small.get(768) == b && small.get(256) == a);
+    small.put(b, 768);
+    small.put(a, 256);
     small.release_all();
     CHECK(g_left == 4096 && g_live.empty());
     return 0;
