@@ -226,13 +226,15 @@ typedef struct {
 int mantra_estimate_batch(mantra_problem* probs, uint32_t count);
 
 /* Autotuner (no counterpart in the paper; it sets how the library runs, not
- * what it computes).  For one graph it times the launch choices of the two
+ * what it computes).  For one graph it times the launch choices of the
  * search kernels on probes -- fixed-r estimates of the graph itself, one per
  * candidate and the same seed for all, each timed by the library's CUDA events
  * -- and keeps the fastest for that graph:
  *   sh / sfm (k_hop): CTA size 256, 512 or 1024 threads (how many samples run
  *     at once per SM, and the vertices a CTA takes per pass) x the next level's
  *     arrivals in shared or in global memory (shared only where they fit);
+ *   RTB and fsfm (k_bfs): CTA size 256, 512 or 1024 x the visited bitmap in
+ *     shared or in global memory, by that kernel's sh search (not reported);
  *   pfm (CTA kernel): CTA size 256 or 512 x the arrival state in shared
  *     memory (as 32-bit arrival slots, or as 16-bit offsets within each
  *     vertex's slots when no vertex has more than 65,534 slots), in global
@@ -242,9 +244,11 @@ int mantra_estimate_batch(mantra_problem* probs, uint32_t count);
  * kernel time by a calibration run of the defaults, between 8 and 64 samples
  * per SM.  Every candidate runs within the same workspace, whose size is bounded by
  * the engine's share of free device memory.  Later calls whose largest graph
- * of that kernel family is g use g's choice.  Results never depend on the choice: sample i
- * draws from Philox counters fixed by (seed, i).  Call it before sharing g
- * between threads; a tuned graph can be tuned again. */
+ * of that kernel family is g use g's choice (sh / sfm ticks of at most two
+ * samples per SM, such as small bootstraps, keep their default shape).
+ * Results never depend on the choice: sample i draws from Philox counters
+ * fixed by (seed, i).  Call it before sharing g between threads; a tuned
+ * graph can be tuned again. */
 typedef struct {
     uint32_t bfs_threads;        /* chosen sh/sfm CTA size */
     uint32_t bfs_bitmap_shared;  /* 1: the per-vertex search state in shared memory */

@@ -31,8 +31,11 @@ using namespace mantra;
 // Launch choices of the search kernels for one graph (mantra_tune); 0 / -1
 // leave the engine's defaults.
 struct Knobs {
-    int bfs_nt = 0;      // sh/sfm CTA size: 256, 512 or 1024
-    int bfs_smem = -1;   // first slots of the next level: 1 shared memory, 0 global
+    int hop_nt = 0;      // k_hop CTA size: 256, 512 or 1024
+    int hop_smem = -1;   // its next level's arrivals: 1 shared memory, 0 global
+    int bfs_nt = 0;      // k_bfs CTA size: 256, 512 or 1024
+    int bfs_smem = -1;   // its visited bitmap: 1 shared memory, 0 global
+    bool sh_on_bfs = false;    // a probe of the two: sh / sfm by k_bfs
     int pfm_nt = 0;      // pfm CTA size: 256 or 512
     int pfm_mode = -1;   // pfm arrival state: 1 shared memory, 0 global, 2 global with the out-edge tiles
                          // staged in shared memory by bulk copies
@@ -961,7 +964,7 @@ double elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
 // Algorithm 2); RTB and fsfm need every state's path count or time: k_bfs.
 // k_hop marks edges in bit 31 of a vertex id.
 bool on_hop(const mantra_graph* G, const Job& j) {
-    return (j.opt == MANTRA_SH || j.opt == MANTRA_SFM) && !j.rtb && G->n < (1u << 31);
+    return (j.opt == MANTRA_SH || j.opt == MANTRA_SFM) && !j.rtb && G->n < (1u << 31) && !G->knobs.sh_on_bfs;
 }
 
 // One line per tick item on stderr (MANTRA_LOG_LAUNCHES): kernel, launch
@@ -1059,6 +1062,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     int rc;
     if ((rc = E.ensure_tables(std::max<uint32_t>(k, 1))) != MANTRA_OK) return rc;
     uint32_t bn = 0, bA = 0, bz = 0, pn = 0, plc = 0, pz = 0;
+    const mantra_graph* gb = nullptr;   // the tick's largest k_bfs graph: its knobs apply
     const mantra_graph* gp = nullptr;   // the tick's largest pfm graph
     uint64_t pwarps = 0, bsamples = 0;
     bool any_b = false, any_h = false, any_p = false, dl = false;
@@ -1095,6 +1099,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         } else {
             any_b = true; bn = std::max(bn, it.G->n); bA = std::max(bA, it.G->A);
             bz = std::max(bz, it.G->dg.max_vslots);
+            if (!gb || it.G->A > gb->A) gb = it.G;
             bsamples += it.job.count;
             dl |= it.job.ob || it.job.rtb;
         }
@@ -1145,14 +1150,15 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     // (two and four samples per SM compete for L2).  A tick of at most two samples
     // per SM wants each of them fast (231 samples: n = 20,000 1024:1 0.33, 512:1
     // 0.42, 256:1 0.61; n = 5,000 0.19, 0.16, 0.21; n = 1,000 0.12, 0.09, 0.09).
-    // mantra_tune's choice for the graph comes first; MANTRA_BFS_NT=256|512|1024 and
-    // MANTRA_BFS_SMEM=0|1 force them.
+    // mantra_tune's choice for the graph comes first in all but such small ticks;
+    // MANTRA_BFS_NT=256|512|1024 and MANTRA_BFS_SMEM=0|1 force them.
     if (any_h) {
         int cls = 0;
         const uint32_t nq = Engine::node_step(hn, &cls);
         auto grid = [&](int nt, int sm) { return E.hop_grid(nt, sm ? nq : 0, INT_MAX); };
         int nt = 1024, sm = 0;
-        if (hsamples <= 2ull * (uint64_t)E.num_sms) {
+        const bool small = hsamples <= 2ull * (uint64_t)E.num_sms;
+        if (small) {
             nt = hn > 12000 ? 1024 : (hn > 1500 ? 512 : 256);
             sm = grid(nt, 1) > 0;
         } else if (grid(256, 1) >= 4 * E.num_sms) {
@@ -1160,7 +1166,7 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
         } else if (grid(512, 1) >= 2 * E.num_sms) {
             nt = 512; sm = 1;
         }
-        if (gh && gh->knobs.bfs_nt) { nt = gh->knobs.bfs_nt; sm = gh->knobs.bfs_smem > 0; }
+        if (gh && !small && gh->knobs.hop_nt) { nt = gh->knobs.hop_nt; sm = gh->knobs.hop_smem > 0; }
         if (const char* env = std::getenv("MANTRA_BFS_NT")) {
             const int v = std::atoi(env);
             nt = v == 1024 ? 1024 : (v == 256 ? 256 : 512);
@@ -1176,10 +1182,12 @@ int run_tick(Engine& E, std::vector<TickItem>& items, bool wide, TickOut* out) {
     // k_bfs CTA shape: 1024 threads for ticks of at most two samples per resident
     // 1024-thread CTA (shorter per-sample latency), else two 512-thread CTAs per
     // SM (measured for sh on the n = 20,000 bursty graph: 1.9 vs 2.7 ms for 231
-    // samples, 42.5 vs 40.4 ms for 26,702); the same variables force them
+    // samples, 42.5 vs 40.4 ms for 26,702), or the shape and bitmap placement that
+    // mantra_tune chose for the graph; the same variables force them
     if (any_b) {
         const bool small = bsamples <= 2ull * (uint64_t)E.bfs_grids[2][E.bfs_rule_smem];
         int nt = small ? 1024 : 512, sm = E.bfs_rule_smem;
+        if (gb && !small && gb->knobs.bfs_nt) { nt = gb->knobs.bfs_nt; sm = gb->knobs.bfs_smem > 0; }
         if (const char* env = std::getenv("MANTRA_BFS_NT")) {
             const int v = std::atoi(env);
             nt = v == 1024 ? 1024 : (v == 256 ? 256 : 512);
@@ -2020,19 +2028,20 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
     };
     const Knobs none{};
     Knobs best{};
-    Knobs search{};      // pfm's defaults on the kernel whose knobs are probed
+    Knobs search{}, bfs{};     // the defaults on the kernels whose knobs are probed
     search.pfm_search = true;
-    auto size_probe = [&](mantra_opt opt) -> int {
+    bfs.sh_on_bfs = true;
+    auto size_probe = [&](mantra_opt opt, const Knobs& k) -> int {
         r = r_lo;
         double ms = 0;
-        const int st = probe(opt, search, &ms);
+        const int st = probe(opt, k, &ms);
         if (st != MANTRA_OK) return st;
         const double per = ms > 0 ? ms / (double)r_lo : 0.0;
         r = per > 0 ? (uint64_t)std::min<double>((double)r_hi, std::max<double>((double)r_lo, 100.0 / per)) : r_hi;
         return MANTRA_OK;
     };
-    // sh/sfm: CTA shape x placement of the first slots (shared memory only where they fit)
-    if ((rc = size_probe(MANTRA_SH)) != MANTRA_OK) { g->knobs = none; return rc; }
+    // sh/sfm (k_hop): CTA shape x placement of the next level's arrivals (shared memory only where they fit)
+    if ((rc = size_probe(MANTRA_SH, none)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->probe_samples = r;
     if ((rc = probe(MANTRA_SH, none, &out->bfs_default_ms)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->bfs_ms = 1e300;
@@ -2040,13 +2049,25 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
         for (int sm = 0; sm < 2; ++sm) {
             if (!E->hop_grid(nt, sm ? g->n : 0, INT_MAX)) continue;
             Knobs k = none;
+            k.hop_nt = nt; k.hop_smem = sm;
+            double ms = 0;
+            if ((rc = probe(MANTRA_SH, k, &ms)) != MANTRA_OK) { g->knobs = none; return rc; }
+            if (ms < out->bfs_ms) { out->bfs_ms = ms; best.hop_nt = nt; best.hop_smem = sm; }
+        }
+    // RTB and fsfm (k_bfs), by its sh search: CTA shape x placement of the visited bitmap
+    if ((rc = size_probe(MANTRA_SH, bfs)) != MANTRA_OK) { g->knobs = none; return rc; }
+    double bfs_ms = 1e300;
+    for (int nt : {256, 512, 1024})
+        for (int sm = 0; sm < 2; ++sm) {
+            if (!E->bfs_grids[Engine::shape_of(nt)][sm]) continue;
+            Knobs k = bfs;
             k.bfs_nt = nt; k.bfs_smem = sm;
             double ms = 0;
             if ((rc = probe(MANTRA_SH, k, &ms)) != MANTRA_OK) { g->knobs = none; return rc; }
-            if (ms < out->bfs_ms) { out->bfs_ms = ms; best.bfs_nt = nt; best.bfs_smem = sm; }
+            if (ms < bfs_ms) { bfs_ms = ms; best.bfs_nt = nt; best.bfs_smem = sm; }
         }
     // pfm (one CTA per sample): CTA shape x arrival-state placement
-    if ((rc = size_probe(MANTRA_PFM)) != MANTRA_OK) { g->knobs = none; return rc; }
+    if ((rc = size_probe(MANTRA_PFM, search)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->pfm_probe_samples = r;
     if ((rc = probe(MANTRA_PFM, search, &out->pfm_default_ms)) != MANTRA_OK) { g->knobs = none; return rc; }
     out->pfm_ms = 1e300;
@@ -2061,13 +2082,13 @@ int mantra_tune(mantra_graph* g, mantra_tune_result* out) {
             if (ms < out->pfm_ms) { out->pfm_ms = ms; best.pfm_nt = nt; best.pfm_mode = sm; }
         }
     g->knobs = best;
-    out->bfs_threads = (uint32_t)best.bfs_nt;
-    out->bfs_bitmap_shared = best.bfs_smem > 0 ? 1u : 0u;
+    out->bfs_threads = (uint32_t)best.hop_nt;
+    out->bfs_bitmap_shared = best.hop_smem > 0 ? 1u : 0u;
     out->pfm_threads = (uint32_t)best.pfm_nt;               // 0: the stream-scan pfm kernel is forced
     out->pfm_state_shared = best.pfm_mode == 1 || best.pfm_mode == 3 ? 1u : 0u;
     out->pfm_staged = best.pfm_mode == 2 ? 1u : 0u;
     out->pfm_state16 = best.pfm_mode == 3 ? 1u : 0u;
-    out->bfs_resident_ctas = best.bfs_nt ? (uint32_t)E->hop_grid(best.bfs_nt, best.bfs_smem > 0 ? g->n : 0, E->hop_regions) : 0u;
+    out->bfs_resident_ctas = best.hop_nt ? (uint32_t)E->hop_grid(best.hop_nt, best.hop_smem > 0 ? g->n : 0, E->hop_regions) : 0u;
     out->pfm_resident_ctas = best.pfm_nt ? (uint32_t)E->pc_grids[best.pfm_nt == 256 ? 0 : 1][best.pfm_mode] : 0u;
     if (!best.pfm_nt) out->pfm_ms = out->pfm_default_ms;
     return MANTRA_OK;
