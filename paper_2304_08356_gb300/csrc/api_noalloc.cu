@@ -89,7 +89,6 @@ extern "C" int mantra_sample_paths_noalloc(const mantra_graph* g, mantra_opt opt
     const bool in_smem = smem + bfs_static_smem(512) + 1024 <= smem_optin;
     BfsWs ws{};
     const size_t region = bfs_region_bytes(n, A, dg->max_vslots, in_smem, false, &ws);
-    ws.nt = 512;
     const size_t head = kHeadBytes + round256(count * 8);
     if (head >= kScratchBytes || region > kScratchBytes - head) return MANTRA_E_INVAL;   // exceeds the fixed scratch
     int grid = (int)std::min<size_t>((size_t)num_sms, (kScratchBytes - head) / region);
@@ -124,8 +123,8 @@ extern "C" int mantra_sample_paths_noalloc(const mantra_graph* g, mantra_opt opt
     ws.base = scratch + head;
     ws.stride = region;
     char* ub = scratch + kUnitOff;
-    if (launch_bfs((const Task*)(scratch + kTaskOff), (const uint64_t*)ub, (const uint32_t*)(ub + 16), (u64*)(ub + 24),
-                   ws, grid, in_smem ? smem : 0, false, st) != cudaSuccess)
+    if (launch_bfs_sampler((const Task*)(scratch + kTaskOff), (const uint64_t*)ub, (const uint32_t*)(ub + 16),
+                           (u64*)(ub + 24), ws, grid, in_smem ? smem : 0, st) != cudaSuccess)
         return MANTRA_E_CUDA;
 
     u64 h[9];

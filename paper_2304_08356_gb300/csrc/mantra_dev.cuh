@@ -1006,6 +1006,8 @@ cudaError_t bfs_configure(size_t smem);
 // sh/sfm: one unit per sample; pfm: one unit per 32 consecutive samples of a task.
 cudaError_t launch_bfs(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
                        const BfsWs& ws, int grid, size_t smem, bool wide, cudaStream_t st);
+cudaError_t launch_bfs_sampler(const Task* tasks, const uint64_t* unit_start, const uint32_t* ntasks, u64* work,
+                               const BfsWs& ws, int grid, size_t smem, cudaStream_t st);
 size_t hop_region_bytes(uint32_t n, uint32_t A, HopWs* ws);
 size_t hop_smem_bytes(int nt, uint32_t n);
 cudaError_t hop_configure(size_t smem);
