@@ -7,7 +7,7 @@ import numpy as np
 import pytest
 
 from oracle import oracle as O
-from test_gpu_sweep import COUNTERS
+from test_gpu_sweep import COUNTERS, _layers
 from test_wave_cut import PART, hub_stream
 
 pytestmark = pytest.mark.gpu
@@ -62,3 +62,44 @@ def test_arrival_in_every_wave_of_a_batch(M, monkeypatch):
     got = g.sample_paths(2, 8, 0, 3000, cap=42)
     assert got == o.samples(2, 8, 0, 3000, cap=42)
     g.free()
+
+
+def _layered(width, depth, lead=0, extra=0):
+    """Complete bipartite steps of width^2 edges after a chain of `lead` edges, which
+    shifts them against the batches of waves; `extra` more edges in the second step."""
+    (u, v, t), n = _layers(width, depth)
+    c = np.arange(lead)
+    u = np.r_[n + c, u.astype(np.int64)]
+    v = np.r_[n + c + 1, v.astype(np.int64)]
+    t = np.r_[c + 1, t.astype(np.int64) + lead]
+    n += lead + 1
+    if extra:
+        u, v, t = np.r_[u, n + np.arange(extra)], np.r_[v, np.full(extra, n + extra)], np.r_[t, np.full(extra, 2 + lead)]
+        n += extra + 1
+    return tuple(x.astype(np.uint32) for x in (u, v, t)), n
+
+
+@pytest.mark.parametrize("width,depth", [(6, 12), (8, 9), (17, 6), (46, 4), (128, 3)])
+def test_steps_of_several_waves(M, monkeypatch, width, depth):
+    """36 to 16,384 edges at one time (2 to 512 waves), every one with in-edges of the
+    same slot: read before any of them is applied."""
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    tri, n = _layered(width, depth)
+    for r in (33, 300):
+        equal(M, tri, n, r)
+
+
+@pytest.mark.parametrize("lead", range(9))
+def test_steps_across_batches(M, monkeypatch, lead):
+    """A step of ten waves that begins in the first to the last wave of a batch."""
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    tri, n = _layered(17, 5, lead=lead)
+    equal(M, tri, n, 300)
+
+
+def test_step_past_the_limit_is_searched(M, monkeypatch):
+    """16,385 edges at one time: the graph has no waves."""
+    monkeypatch.setenv("MANTRA_PFM_KERNEL", "sweep")
+    tri, n = _layered(128, 3, extra=1)
+    assert np.unique(tri[2], return_counts=True)[1].max() == 16385
+    equal(M, tri, n, 300, swept=False)
