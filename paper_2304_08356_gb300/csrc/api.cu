@@ -124,9 +124,12 @@ int upload_store(const StoreHost& H, mantra_graph* G, Engine& E, cudaStream_t st
     dst[SA_OUT_LOFF] = &loff_words;
     size_t total = 0;
     for (int k = 0; k < SA_COUNT; ++k) total += al256((H.len[k] + 1) * 4);
-    // filled on the device: the edges' head and continuation, the in-edges' out-CSR
-    // index, the edges' usable slots, and the out-rows cut at up to 32 times (as many as the mean row has
-    // edges, so that the directory is no larger than the edge arrays)
+    // filled on the device, for k_hop: the edges' head and continuation, the in-edges'
+    // out-CSR index, the edges' usable slots, and the out-rows cut at up to 32 times (as
+    // many as the mean row has edges, so that the directory is no larger than the edge
+    // arrays).  A device without room for them (16 to 32 B an edge, the store 54) holds
+    // the store alone: sh and sfm then run on k_bfs.
+    const size_t store = total;
     uint32_t nb = 1;
     while (nb < 32 && (uint64_t)nb * H.n < H.m) nb *= 2;
     const size_t o_vn = total;
@@ -140,6 +143,8 @@ int upload_store(const StoreHost& H, mantra_graph* G, Engine& E, cudaStream_t st
     const size_t o_dt = total;
     total += al256(32 * 4);
     G->dmem = graph_block(E, total, false);
+    const bool maps = G->dmem != nullptr;
+    if (!maps) G->dmem = graph_block(E, total = store, false);
     if (!G->dmem) return MANTRA_E_NOMEM;
     G->b_dmem = total;
     size_t off = 0;
@@ -149,18 +154,20 @@ int upload_store(const StoreHost& H, mantra_graph* G, Engine& E, cudaStream_t st
         *dst[k] = (const uint32_t*)p;
         off += al256((H.len[k] + 1) * 4);
     }
-    DirTimes dt{};
-    for (uint32_t j = 1; j < nb; ++j) dt.t[j] = H.arr[SA_ST_T][(size_t)j * H.m / nb];   // m > n here
-    char* base = (char*)G->dmem;
     G->dg.n = H.n; G->dg.m = H.m; G->dg.A = H.A;
-    G->dg.out_vn = (const uint2*)(base + o_vn);
-    G->dg.in_out = (const uint32_t*)(base + o_io);
-    G->dg.out_pend = (const uint32_t*)(base + o_pe);
-    G->dg.dir = (const uint2*)(base + o_dir);
-    G->dg.dir_t = (const uint32_t*)(base + o_dt);
-    G->dg.dir_n = nb;
-    CU(launch_edge_maps(G->dg, dt, (uint2*)(base + o_vn), (uint32_t*)(base + o_io), (uint32_t*)(base + o_pe),
-                        (uint2*)(base + o_dir), (uint32_t*)(base + o_dt), st));
+    if (maps) {
+        DirTimes dt{};
+        for (uint32_t j = 1; j < nb; ++j) dt.t[j] = H.arr[SA_ST_T][(size_t)j * H.m / nb];   // m > n here
+        char* base = (char*)G->dmem;
+        G->dg.out_vn = (const uint2*)(base + o_vn);
+        G->dg.in_out = (const uint32_t*)(base + o_io);
+        G->dg.out_pend = (const uint32_t*)(base + o_pe);
+        G->dg.dir = (const uint2*)(base + o_dir);
+        G->dg.dir_t = (const uint32_t*)(base + o_dt);
+        G->dg.dir_n = nb;
+        CU(launch_edge_maps(G->dg, dt, (uint2*)(base + o_vn), (uint32_t*)(base + o_io), (uint32_t*)(base + o_pe),
+                            (uint2*)(base + o_dir), (uint32_t*)(base + o_dt), st));
+    }
     CU(cudaStreamSynchronize(st));
     G->dg.out_loff = reinterpret_cast<const unsigned short*>(loff_words);
     G->n = H.n; G->m = H.m; G->A = H.A; G->n_uedge = H.n_uedge;
@@ -190,6 +197,7 @@ int build_waves(mantra_graph* G, size_t smem_optin, Engine& E, cudaStream_t st) 
     const uint32_t m = G->m;
     const char* env = std::getenv("MANTRA_PFM_KERNEL");
     const bool force = env && std::strcmp(env, "sweep") == 0;
+    if (!G->dg.dir_t) return MANTRA_OK;                      // k_sweep_order's times; the device is full
     if (m < (force ? 1u : 1u << 16) || !(force || few_choices(G)) || sweep_smem_bytes(G->n) + sweep_static_smem() + 1024 > smem_optin) return MANTRA_OK;
     const size_t bytes = wave_tmp_bytes(m, G->A);
     char* tmp = (char*)graph_block(E, bytes, true);
@@ -962,9 +970,10 @@ double elapsed_ms(cudaEvent_t a, cudaEvent_t b) {
 
 // Whether a 64-bit sh / sfm search runs on k_hop (trk and ob estimates,
 // Algorithm 2); RTB and fsfm need every state's path count or time: k_bfs.
-// k_hop marks edges in bit 31 of a vertex id.
+// k_hop marks edges in bit 31 of a vertex id, and needs its maps of the edges.
 bool on_hop(const mantra_graph* G, const Job& j) {
-    return (j.opt == MANTRA_SH || j.opt == MANTRA_SFM) && !j.rtb && G->n < (1u << 31) && !G->knobs.sh_on_bfs;
+    return (j.opt == MANTRA_SH || j.opt == MANTRA_SFM) && !j.rtb && G->n < (1u << 31) && G->dg.out_vn &&
+           !G->knobs.sh_on_bfs;
 }
 
 // One line per tick item on stderr (MANTRA_LOG_LAUNCHES): kernel, launch
@@ -1791,7 +1800,7 @@ struct Server {
                 if (G->dg.n_scan) w.scan_n = std::max(w.scan_n, G->n);
             } else {
                 w.n = std::max(w.n, G->n); w.A = std::max(w.A, G->A); w.vslots = std::max(w.vslots, G->dg.max_vslots);
-                w.full = w.full || r->p.estimator == 2 || r->p.opt == MANTRA_FSFM;
+                w.full = w.full || r->p.estimator == 2 || r->p.opt == MANTRA_FSFM || !G->dg.out_vn;
             }
         };
         for (const Request* r : active) add(r);

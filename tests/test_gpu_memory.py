@@ -165,3 +165,47 @@ def test_idle_workspaces_make_room(M):
         assert np.array_equal(big.estimate(opt, 0.05, 0.1, 3, fixed_r=2000)[1], want[opt])
     big.free()
     other.free()
+
+
+STORE_ONLY = """
+import sys
+import numpy as np, torch
+sys.path.insert(0, "tests")
+import test_gpu_memory as T
+from paper_2304_08356_gb300 import mantra as M, synth
+M.Graph(*T.few_heads(m=70000), n=200).free()
+n, m = 100000, 2000000
+tri = synth.chung_lu_uniform_t(n=n, m=m, seed=1)
+fill = T.Filler(54 * m + 16 * n + (14 << 20))      # 54 B an edge: the store; 28 more: its maps for k_hop
+g = M.Graph(*tri, n=n)
+fill.release()
+h = M.Graph(*tri, n=n)
+for opt, est in ((0, 0), (0, 1), (1, 0), (2, 0), (3, 0)):
+    print("opt", opt, file=sys.stderr, flush=True)
+    a = g.estimate(opt, 0.05, 0.1, 3, fixed_r=300, estimator=est)
+    print("other", file=sys.stderr, flush=True)
+    b = h.estimate(opt, 0.05, 0.1, 3, fixed_r=300, estimator=est)
+    assert np.array_equal(a[1], b[1]) and a[1].sum() > 0
+    assert all(a[2][k] == b[2][k] for k in ("rade_num", "sum_int_len", "max_hits"))
+st = [x.temporal_stats(0, 0.1, 5, r_override=20)[1] for x in (g, h)]
+assert np.array_equal(*st)
+print("same")
+"""
+
+
+def test_load_with_room_for_the_store_alone(M):
+    """In a fresh process: a graph whose maps for k_hop find no room loads, and its sh
+    and sfm samples run on k_bfs with the same results."""
+    import os
+    import re
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", STORE_ONLY], capture_output=True, text=True, cwd=root,
+                       env=dict(os.environ, MANTRA_LOG_LAUNCHES="1"))
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-3000:]
+    parts = re.split(r"^opt (\d)$", r.stderr, flags=re.M)
+    for opt, text in zip(parts[1::2], parts[2::2]):
+        mine, other = text.split("other\n")[:2]
+        if opt in "01":
+            assert "kernel=k_bfs" in mine and "kernel=k_hop" not in mine and "kernel=k_hop" in other
