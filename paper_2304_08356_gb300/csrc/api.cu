@@ -322,8 +322,8 @@ struct Engine {
     // threads, arrivals in global memory); shapes 0 = 256, 1 = 512, 2 = 1024
     // threads; the arrivals in shared memory are sized by the tick's graphs
     // (hop_nsm: their largest node count, rounded up)
-    char* hop_mem = nullptr; HopWs hws{}; uint32_t hop_n = 0, hop_A = 0;
-    int hop_regions = 0, hop_want = 0;     // regions allocated, and wanted then
+    char* hop_mem = nullptr; size_t hop_bytes = 0; HopWs hws{}; uint32_t hop_n = 0, hop_A = 0;
+    int hop_regions = 0, hop_want = 0;     // regions of the present layout, and wanted for it
     std::map<uint64_t, int> hop_occ;       // (shape, shared nodes) -> CTAs per SM
     int tick_hop_nt = 256, tick_hop_sm = 0, tick_hop_cls = 0;
     uint32_t tick_hop_n = 0;
@@ -438,7 +438,7 @@ struct Engine {
         drop(tick_p && tick_cta, &pc_mem);
         drop(tick_s, &sw_mem);
         drop(tick_n, &sc_mem);
-        if (!hop_mem) { hop_n = hop_A = 0; hop_regions = hop_want = 0; }
+        if (!hop_mem) { hop_n = hop_A = 0; hop_regions = hop_want = 0; hop_bytes = 0; }
         if (!bfs_mem) { bfs_n = bfs_A = bfs_z = 0; bfs_dl = false; }
         if (!pfm_mem) { pfm_n = pfm_lcap = 0; pfm_warps = 0; }
         if (!pc_mem) { pc_n = pc_cb = 0; }
@@ -563,26 +563,39 @@ struct Engine {
     // sh/sfm level search: a region per CTA of the largest resident grid of any shape
     // while that is at most 4 GB, else per CTA that the tick runs (n = 10^6 and m =
     // 2*10^7: 152 CTAs and 41 GB, 160 GB for all shapes); at most 45 % of free memory
-    // (k_bfs and the pfm kernels may need theirs beside it).
+    // (k_bfs and the pfm kernels may need theirs beside it).  Regions hold the largest
+    // graphs seen; where that takes more memory than there is now, they are laid out
+    // for the tick's graphs alone, within the present allocation if it suffices (a
+    // layout is cleared first: 6 ms for those 41 GB, whose tick takes ten times that).
     int ensure_hop(uint32_t n, uint32_t A, int ctas) {
         if (hop_mem && n <= hop_n && A <= hop_A && ctas <= hop_want) return MANTRA_OK;
-        n = std::max(n, hop_n);
-        A = std::max(A, hop_A);
-        int want = std::max(ctas, hop_want);
-        if (hop_mem) { cudaStreamSynchronize(sa); cudaFree(hop_mem); hop_mem = nullptr; }
-        const size_t region = hop_region_bytes(n, A, &hws);
         int all = 1;
         for (int nt : {256, 512, 1024}) all = std::max(all, hop_grid(nt, 0, INT_MAX));
-        if ((size_t)all * region <= (size_t)4 << 30) want = all;
-        const int grid = regions_for(want, region, 0.45);
-        if (!alloc(&hop_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+        constexpr size_t small = (size_t)4 << 30;
+        uint32_t ln = std::max(n, hop_n), lA = std::max(A, hop_A);
+        size_t region = 0;
+        int want = 0;
+        for (bool again : {true, false}) {
+            region = hop_region_bytes(ln, lA, &hws);
+            want = (size_t)all * region <= small ? all : ctas;
+            if (!again || (size_t)want * region <= std::max(small, hop_bytes)) break;
+            ln = n; lA = A;
+        }
+        int grid = want;
+        if ((size_t)want * region > hop_bytes) {
+            if (hop_mem) { cudaStreamSynchronize(sa); cudaFree(hop_mem); hop_mem = nullptr; hop_bytes = 0; }
+            grid = regions_for(want, region, 0.45);
+            if (!alloc(&hop_mem, (size_t)grid * region)) return MANTRA_E_NOMEM;
+            hop_bytes = (size_t)grid * region;
+        }
+        invalidate_graph();
+        hop_n = hop_A = 0;
         CU(cudaMemsetAsync(hop_mem, 0, (size_t)grid * region, sa));
         hws.base = hop_mem;
         hws.stride = region;
         hop_regions = grid;
         hop_want = want;
-        hop_n = n; hop_A = A;
-        invalidate_graph();
+        hop_n = ln; hop_A = lA;
         return MANTRA_OK;
     }
 

@@ -209,3 +209,39 @@ def test_load_with_room_for_the_store_alone(M):
         mine, other = text.split("other\n")[:2]
         if opt in "01":
             assert "kernel=k_bfs" in mine and "kernel=k_hop" not in mine and "kernel=k_hop" in other
+
+
+LAYOUTS = """
+import numpy as np, torch
+from paper_2304_08356_gb300 import mantra as M, synth
+a = M.Graph(*synth.chung_lu_bursty(n=2000, m=40000, seed=3))
+b = M.Graph(*synth.chung_lu_uniform_t(n=300000, m=6000000, seed=4), n=300000)
+free = lambda: torch.cuda.mem_get_info()[0]
+def run(g, r):
+    res = [g.estimate(0, 0.05, 0.1, 3, fixed_r=r)[1:] for _ in range(5)]
+    return res[0][0], min(i["kernel_ms"] for _, i in res)
+before = free()
+ha, ms = run(a, 20000)
+print("small", before - free())
+hb, _ = run(b, 500)
+print("large", before - free())
+for _ in range(2):
+    h, ms2 = run(a, 20000)
+    assert np.array_equal(h, ha) and ms2 < 1.5 * ms, (ms, ms2)
+    assert np.array_equal(run(b, 500)[0], hb)
+print("end", before - free())
+"""
+
+
+def test_hop_workspace_fits_the_graphs(M):
+    """In a fresh process: a small graph's many CTAs and then a large graph's regions
+    do not multiply, and the small graph's calls are as fast after the large one's."""
+    import os
+    import re
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", LAYOUTS], capture_output=True, text=True, cwd=root)
+    assert r.returncode == 0, r.stderr[-3000:]
+    held = {k: int(x) for k, x in re.findall(r"(\w+) (\d+)", r.stdout)}
+    assert held["large"] < 20 << 30 and held["end"] <= held["large"] + (64 << 20), held
