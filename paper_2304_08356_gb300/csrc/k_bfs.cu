@@ -1,6 +1,6 @@
 // (*)-temporal BFS with a path count for every state: the RTB estimator and the
-// foremost-first order (fsfm), the 128-bit re-runs of every sh / sfm search, and
-// the allocation-free sampler (other sh / sfm searches: k_hop.cu).  For the
+// foremost-first order (fsfm), the 128-bit re-runs of every sh / sfm search,
+// samples past k_hop's caps, and the allocation-free sampler (other sh / sfm searches: k_hop.cu).  For the
 // shortest (sh) and shortest-foremost (sfm)
 // optimalities (paper Sec. 3 Def. 1; running-time theorem of Sec. 4.4), the
 // backward path draw of the temporal Riondato-Kornaropoulos estimator

@@ -29,7 +29,9 @@
 // L2 accesses (list entry, arrival and row directory, a few probes of the row,
 // the edge window, the heads' arrivals) with five block barriers; about 170,000
 // warp instructions per sample on the bursty 20,000-node graph, 0.3 issued per
-// scheduler and cycle, DRAM at 18 % and L2 at 33 % of their peaks.  The loads of
+// scheduler and cycle, DRAM at 18 % and L2 at 33 % of their peaks (with the arrivals
+// in shared memory 131,000 instructions, DRAM 14 %, L2 24 %, 8.7 of 23 cycles
+// per instruction at barriers).  The loads of
 // four edge windows and two vertices per thread are issued together (one at a
 // time: 40 against 10 ms with the arrivals in global memory).  22,000 sh samples
 // on that graph take 7.2 ms; the search with per-state path counts and a visited
